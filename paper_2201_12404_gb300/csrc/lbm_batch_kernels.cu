@@ -54,7 +54,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int* er
 #endif
 template <int BX, int BY, typename S, typename R, typename A>
 __global__ void __launch_bounds__(BX * BY, sizeof(R) == 4 ? LBM_BATCH_MINBLOCKS_F32 : 1) batch_persistent_kernel(BatchArgs a) {
-  __shared__ __align__(128) Two<A> s_aux[Halo<2, BX, BY, 1>::HN];
+  __shared__ __align__(128) Two<A> s_aux[QTileShape<2, BX, BY, 1>::HX * QTileShape<2, BX, BY, 1>::HY];
   extern __shared__ __align__(128) unsigned char smem_dyn[];
   R* s_h = (R*)smem_dyn;
   for (int s = 0; s < a.nsteps; ++s) {
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(BX * BY, sizeof(R) == 4 ? LBM_BATCH_MINBLOCKS_
 template <int BX, int BY, typename S, typename R, typename A>
 BatchVariant variant() {
   return BatchVariant{BX, BY, (const void*)&batch_persistent_kernel<BX, BY, S, R, A>,
-                      (size_t)Lattice<2>::Q * BX * BY * sizeof(R)};
+                      collide_dyn_smem<2, R>(BX * BY)};
 }
 
 int batch_variants(int precision, const BatchVariant** out) {

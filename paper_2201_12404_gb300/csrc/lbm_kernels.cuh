@@ -45,8 +45,9 @@ __device__ __forceinline__ void moments_eos_node(const DevDomain& d, int x, int 
   if (x >= d.nx || y >= d.ny || z >= d.nz) return;
   R f[Q];
   gather<D, P, S, R>(d, x, y, z, f);
-  R rho, j[3], Pi[6];
-  moments<D, R>(f, rho, j, Pi);
+  NodeMoments<R> m;
+  row_moments<D, R>(f, m);
+  const R rho = m.rho, j[3] = {m.jx, m.jy, m.jz};
   if (!(rho > (R)0) || !(rho < (R)INFINITY)) atomicOr(d.flags, 1u);
 
   A* aux = (A*)d.aux;
@@ -62,9 +63,9 @@ __device__ __forceinline__ void moments_eos_node(const DevDomain& d, int x, int 
   const int gz = D == 3 ? ghost_of(z, d.nz, d.wall_lo[2], d.wall_hi[2], &wall) : -1;
   if (gx < 0 && gy < 0 && gz < 0) return;
 #pragma unroll 1
-  for (int m = 1; m < (1 << D); ++m) {
-    if (((m & 1) && gx < 0) || ((m & 2) && gy < 0) || ((m & 4) && gz < 0)) continue;
-    const int cx = (m & 1) ? gx : x + 2, cy = (m & 2) ? gy : y + 2, cz = D == 3 ? ((m & 4) ? gz : z + 2) : 0;
+  for (int k = 1; k < (1 << D); ++k) {
+    if (((k & 1) && gx < 0) || ((k & 2) && gy < 0) || ((k & 4) && gz < 0)) continue;
+    const int cx = (k & 1) ? gx : x + 2, cy = (k & 2) ? gy : y + 2, cz = D == 3 ? ((k & 4) ? gz : z + 2) : 0;
     a2[bc_pnode(d, (long long)cx + (long long)d.px * ((long long)cy + (long long)d.py * cz))] = pair;
   }
 }
@@ -88,8 +89,16 @@ __global__ void __launch_bounds__(256) aux_density_kernel(DevDomain d, const dou
   ((Two<A>*)d.aux)[pn] = two<A>((A)rho, (A)psi_of<R>(d, rho));
 }
 
+// Resident blocks per SM asked of the register allocator: 16 of 64 threads, 64
+// registers, in the D3Q27 float32 and float16 kernels (256x256x128 impact in float16
+// deviations, passes 1 + 1b: 351 us, 372 before, at 76 registers in odd steps).
+#ifndef LBM_K1_MINBLOCKS_F32
+#define LBM_K1_MINBLOCKS_F32 16
+#endif
 template <int D, int P, typename S, typename R, typename A>
-__global__ void __launch_bounds__(256) moments_eos_kernel(DevDomain d) {
+__global__ void __launch_bounds__(Blocks<D, R>::bx * Blocks<D, R>::by * Blocks<D, R>::bz,
+                                  D == 3 && sizeof(R) == 4 ? LBM_K1_MINBLOCKS_F32 : 1)
+moments_eos_kernel(DevDomain d) {
   moments_eos_node<D, P, S, R, A>(d, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y,
                                   blockIdx.z * blockDim.z + threadIdx.z);
 }

@@ -128,11 +128,9 @@ inline bool make_aux_map(CUtensorMap* map, const DevDomain& d, int D, size_t ele
 }
 
 // Tensor map over the q_a planes (element offset 2 PN of d.aux, one plane per
-// axis): a (px, py[, pz], D) tensor with a box of (Blocks::bx + 4, Blocks::by + 2
-// [, Blocks::bz + 2], 1), which holds q_a at the tile's nodes and their +-1
-// neighbours along every axis (x starts 2 nodes early so that the box starts on a
-// 16-byte boundary).
-inline bool make_q_map(CUtensorMap* map, const DevDomain& d, int D, size_t elem_bytes, const char** why) {
+// axis): a (px, py[, pz], D) tensor with a box of `tile` values of one plane.
+inline bool make_q_map(CUtensorMap* map, const DevDomain& d, int D, size_t elem_bytes, const cuuint32_t tile[3],
+                       const char** why) {
   const tensor_map_encode_fn encode = tensor_map_encoder(why);
   if (!encode) return false;
   const cuuint64_t e = elem_bytes;
@@ -141,13 +139,13 @@ inline bool make_q_map(CUtensorMap* map, const DevDomain& d, int D, size_t elem_
   const cuuint32_t rank = (cuuint32_t)D + 1;
   dims[0] = d.px; dims[1] = d.py;
   strides[0] = d.px * e;
-  box[0] = (D == 3 ? Blocks<3>::bx : Blocks<2>::bx) + 4;
-  box[1] = (D == 3 ? Blocks<3>::by : Blocks<2>::by) + 2;
+  box[0] = tile[0];
+  box[1] = tile[1];
   if (D == 3) {
     dims[2] = d.pz; dims[3] = 3;
     strides[1] = (cuuint64_t)d.px * d.py * e;
     strides[2] = (cuuint64_t)d.PN * e;
-    box[2] = Blocks<3>::bz + 2; box[3] = 1;
+    box[2] = tile[2]; box[3] = 1;
   } else {
     dims[2] = 2;
     strides[1] = (cuuint64_t)d.PN * e;
@@ -190,15 +188,32 @@ inline void qtile_box(cuuint32_t box[3]) {
   box[0] = T::HX; box[1] = T::HY; box[2] = T::HZ;
 }
 
+// The q box of axis a for a tile of pass 2.
+template <int D, typename R>
+inline void qbox_tile(int a, cuuint32_t box[3]) {
+  using B = Blocks<D, R>;
+  using H = QBox<D, B::bx, B::by, B::bz>;
+  box[0] = H::X; box[1] = H::Y(a); box[2] = H::Z(a);
+}
+
 inline bool make_tile_maps(TileMaps* m, const DevDomain& d, int D, size_t elem_bytes, const char** why) {
   // pass 1b: a QTile tile with a 2-node halo
-  cuuint32_t qbox[3];
+  cuuint32_t box[3];
   if (D == 3) {
-    if (elem_bytes == 4) qtile_box<3, 8>(qbox); else qtile_box<3, 16>(qbox);
+    if (elem_bytes == 4) qtile_box<3, 8>(box); else qtile_box<3, 16>(box);
   } else {
-    if (elem_bytes == 4) qtile_box<2, 8>(qbox); else qtile_box<2, 16>(qbox);
+    if (elem_bytes == 4) qtile_box<2, 8>(box); else qtile_box<2, 16>(box);
   }
-  return make_aux_map(&m->aux_q, d, D, elem_bytes, qbox, why) && make_q_map(&m->q, d, D, elem_bytes, why);
+  if (!make_aux_map(&m->aux_q, d, D, elem_bytes, box, why)) return false;
+  for (int a = 0; a < D; ++a) {
+    if (D == 3) {
+      if (elem_bytes == 4) qbox_tile<3, float>(a, box); else qbox_tile<3, double>(a, box);
+    } else {
+      if (elem_bytes == 4) qbox_tile<2, float>(a, box); else qbox_tile<2, double>(a, box);
+    }
+    if (!make_q_map(&m->q[a], d, D, elem_bytes, box, why)) return false;
+  }
+  return true;
 }
 
 // Final fixed-order reduction of the diagnostic partial sums (lbm_d2q9.cu).
