@@ -325,24 +325,22 @@ double bisect_p(const EosCoeffs& e, double target, double lo, double hi) {
   return 0.5 * (lo + hi);
 }
 
-// Pass 1 for the current state, then a block-partial maximum (field 4 of the
-// [block][5] layout, at most N blocks) reduced by diag_final_kernel; *out = the maximum.
+// Pass 1 for the current state, then block maxima (partial(buf, stream), which returns
+// their number and launches nothing for a null buffer) and their maximum in *out.
 template <typename Partial>
 lbm_status reduce_max(lbm_handle h, Partial partial, double* out) {
   lbm_status st = refresh_aux(h);
   if (st != LBM_OK) return st;
-  const long long nblk = (h->dev.N + 255) / 256;
+  const long long nb = partial(nullptr);
   double* buf = nullptr;
-  LBM_CUDA(h, scratch_alloc(h, &buf, (size_t)(nblk * 5 + 5) * sizeof(double)));
-  const int nb = partial(buf);
-  lbm::launch_diag_final(buf, nb, buf + nblk * 5, h->stream);
+  LBM_CUDA(h, scratch_alloc(h, &buf, (size_t)(nb + 1) * sizeof(double)));
+  partial(buf);
+  lbm::launch_max_final(buf, nb, buf + nb, h->stream);
   h->launches += 2;
   LBM_CUDA(h, cudaGetLastError());
-  double res[5];
-  LBM_CUDA(h, cudaMemcpyAsync(res, buf + nblk * 5, sizeof(res), cudaMemcpyDeviceToHost, h->stream));
+  LBM_CUDA(h, cudaMemcpyAsync(out, buf + nb, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   LBM_CUDA(h, cudaFreeAsync(buf, h->stream));
   LBM_CUDA(h, cudaStreamSynchronize(h->stream));
-  *out = res[4];
   return LBM_OK;
 }
 
@@ -640,7 +638,7 @@ lbm_status lbm_read_macroscopic(lbm_handle h, double* rho, double* ux, double* u
   const size_t nb = (size_t)h->dev.N * sizeof(double);
   double* buf = nullptr;
   LBM_CUDA(h, scratch_alloc(h, &buf, nb * (1 + D)));
-  h->ops->macroscopic(h->dev, h->parity, buf, buf + h->dev.N, h->stream);
+  h->ops->macroscopic(h->dev, h->maps, buf, buf + h->dev.N, h->stream);
   h->launches += 1;
   LBM_CUDA(h, cudaGetLastError());
   LBM_CUDA(h, cudaMemcpyAsync(rho, buf, nb, cudaMemcpyDeviceToHost, h->stream));
@@ -710,7 +708,7 @@ lbm_status lbm_write_populations(lbm_handle h, const double* host, size_t count)
 
 lbm_status lbm_read_diag(lbm_handle h, double* mass, double* momentum3, double* max_u, double* gamma_field) {
   LBM_LIVE(h);
-  const long long nblk = (h->dev.N + 255) / 256;
+  const int nblk = lbm::diag_blocks();
   double* buf = nullptr;
   LBM_CUDA(h, scratch_alloc(h, &buf, (size_t)(nblk * 5 + 5) * sizeof(double)));
   int nb = h->ops->diag_partial(h->dev, h->parity, buf, h->stream);
@@ -739,7 +737,7 @@ lbm_status lbm_read_diag(lbm_handle h, double* mass, double* momentum3, double* 
 lbm_status lbm_max_speed(lbm_handle h, double* max_u) {
   LBM_LIVE(h);
   if (!max_u) return fail(h, LBM_ERR_INVALID_ARG, "max_u is NULL");
-  return reduce_max(h, [&](double* buf) { return h->ops->max_speed_partial(h->dev, h->parity, buf, h->stream); }, max_u);
+  return reduce_max(h, [&](double* buf) { return h->ops->speed_partial(h->dev, h->maps, buf, h->stream); }, max_u);
 }
 
 lbm_status lbm_interface_width(lbm_handle h, double* width, double* max_grad) {

@@ -12,16 +12,26 @@ struct Launch {
   using B = Blocks<D, R>;
   static dim3 block() { return dim3(B::bx, B::by, B::bz); }
   static dim3 tile_grid(const DevDomain& d) {
-    return dim3((d.nx + B::bx - 1) / B::bx, (d.ny + B::by - 1) / B::by, (d.nz + B::bz - 1) / B::bz);
+    const unsigned ty = (d.ny + B::by - 1) / B::by;
+    const unsigned gx = (d.nx + B::bx - 1) / B::bx;
+    if (D == 2) {  // tile_y
+      const unsigned gz = (ty + 65534) / 65535;
+      return dim3(gx, (ty + gz - 1) / gz, gz);
+    }
+    return dim3(gx, ty, (d.nz + B::bz - 1) / B::bz);
   }
   static void moments_eos(const DevDomain& d, int parity, cudaStream_t s) {
     if (parity == 0) moments_eos_kernel<D, 0, S, R, A><<<tile_grid(d), block(), 0, s>>>(d);
     else moments_eos_kernel<D, 1, S, R, A><<<tile_grid(d), block(), 0, s>>>(d);
   }
-  static void qflux(const DevDomain& d, const TileMaps& maps, cudaStream_t s) {
-    using T = QTile<D, 2 * sizeof(A)>;
+  using QT = QTile<D, 2 * sizeof(A)>;
+  static dim3 qflux_grid(const DevDomain& d) {
+    return dim3((d.nx + QT::EX - 1) / QT::EX, (d.ny + QT::EY - 1) / QT::EY, (d.nz + QT::EZ - 1) / QT::EZ);
+  }
+  template <int kMode>
+  static void qflux_launch(const DevDomain& d, const TileMaps& maps, double* out0, double* out1, cudaStream_t s) {
     constexpr size_t smem = qflux_dyn_smem<D, A>();
-    auto k = qflux_tile_kernel<D, R, A>;
+    auto k = qflux_tile_kernel<D, R, A, kMode>;
     constexpr int kMaxDev = 64;
     static bool opted_in[kMaxDev] = {};
     int dev = 0;
@@ -30,8 +40,10 @@ struct Launch {
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (dev >= 0 && dev < kMaxDev) opted_in[dev] = true;
     }
-    const dim3 grd((d.nx + T::EX - 1) / T::EX, (d.ny + T::EY - 1) / T::EY, (d.nz + T::EZ - 1) / T::EZ);
-    k<<<grd, dim3(T::TX, T::TY), smem, s>>>(d, maps);
+    k<<<qflux_grid(d), dim3(QT::TX, QT::TY), smem, s>>>(d, maps, out0, out1);
+  }
+  static void qflux(const DevDomain& d, const TileMaps& maps, cudaStream_t s) {
+    qflux_launch<kQfluxStep>(d, maps, nullptr, nullptr, s);
   }
   static void collide_stream(const DevDomain& d, const TileMaps& maps, int parity, cudaStream_t s) {
     constexpr size_t smem = collide_dyn_smem<D, R>(B::bx * B::by * B::bz);
@@ -69,39 +81,47 @@ struct Launch {
     if constexpr (DevStorage<S>::value) canonical_density_kernel<D><<<blocks1d(d), 256, 0, s>>>(d, in);
     canonical_write_kernel<D, S><<<blocks1d(d), 256, 0, s>>>(d, in);
   }
-  static void macroscopic(const DevDomain& d, int parity, double* rho, double* u, cudaStream_t s) {
-    macroscopic_kernel<D, S, R, A><<<blocks1d(d), 256, 0, s>>>(d, parity, rho, u);
+  static void macroscopic(const DevDomain& d, const TileMaps& maps, double* rho, double* u, cudaStream_t s) {
+    qflux_launch<kQfluxFields>(d, maps, rho, u, s);
   }
   static void bare_velocity(const DevDomain& d, const double* rho, double* u, cudaStream_t s) {
     bare_velocity_kernel<D, R, A><<<blocks1d(d), 256, 0, s>>>(d, rho, u);
   }
+  // Tiles of 32 x 8 nodes for the grid-stride readings, and the blocks that walk them.
+  struct Tiles {
+    int x, y, n, blocks;
+    explicit Tiles(const DevDomain& d) : x((d.nx + 31) / 32), y((d.ny + 7) / 8), n(x * y * d.nz), blocks(n < kDiagBlocks ? n : kDiagBlocks) {}
+  };
   static int diag_partial(const DevDomain& d, int parity, double* partial, cudaStream_t s) {
-    diag_partial_kernel<D, S><<<blocks1d(d), 256, 0, s>>>(d, parity, partial);
-    return (int)blocks1d(d);
+    const Tiles t(d);
+    diag_partial_kernel<D, S><<<t.blocks, dim3(32, 8), 0, s>>>(d, parity, t.x, t.y, t.n, partial);
+    return t.blocks;
   }
-  static int max_speed_partial(const DevDomain& d, int parity, double* partial, cudaStream_t s) {
-    max_speed_partial_kernel<D, S, R, A><<<blocks1d(d), 256, 0, s>>>(d, parity, partial);
-    return (int)blocks1d(d);
+  static long long speed_partial(const DevDomain& d, const TileMaps& maps, double* partial, cudaStream_t s) {
+    const dim3 g = qflux_grid(d);
+    if (partial) qflux_launch<kQfluxSpeed>(d, maps, partial, nullptr, s);
+    return (long long)g.x * g.y * g.z;
   }
   static void drop_on_film(const DevDomain& d, const lbm_drop_on_film& g, double rho_l, double rho_v, double* rho,
                            double* u, cudaStream_t s) {
     drop_on_film_kernel<D><<<blocks1d(d), 256, 0, s>>>(d, g.radius, g.film, g.gap, g.speed, g.width, g.noise,
                                                        (unsigned long long)g.seed, rho_l, rho_v, rho, u);
   }
-  static int grad_partial(const DevDomain& d, double* partial, cudaStream_t s) {
-    grad_partial_kernel<D, A><<<blocks1d(d), 256, 0, s>>>(d, partial);
-    return (int)blocks1d(d);
+  static long long grad_partial(const DevDomain& d, double* partial, cudaStream_t s) {
+    const Tiles t(d);
+    if (partial) grad_partial_kernel<D, A><<<t.blocks, dim3(32, 8), 0, s>>>(d, t.x, t.y, t.n, partial);
+    return t.blocks;
   }
-  static int crown_partial(const DevDomain& d, int layer, double rho_mid, double* partial, cudaStream_t s) {
+  static long long crown_partial(const DevDomain& d, int layer, double rho_mid, double* partial, cudaStream_t s) {
     const long long nl = D == 3 ? (long long)d.nx * d.ny : d.nx;
     const unsigned nb = (unsigned)((nl + 255) / 256);
-    crown_partial_kernel<D, A><<<nb, 256, 0, s>>>(d, layer, rho_mid, partial);
-    return (int)nb;
+    if (partial) crown_partial_kernel<D, A><<<nb, 256, 0, s>>>(d, layer, rho_mid, partial);
+    return (long long)nb;
   }
   static Ops table() {
     return Ops{D, Lattice<D>::Q, sizeof(S), sizeof(A), &moments_eos, &qflux, &collide_stream, &init_equilibrium, &aux_density,
                &canonical_read, &canonical_write, &canonical_window, &macroscopic, &bare_velocity, &diag_partial,
-               &max_speed_partial, &drop_on_film, &grad_partial, &crown_partial};
+               &speed_partial, &drop_on_film, &grad_partial, &crown_partial};
   }
 };
 

@@ -14,6 +14,8 @@
 //                                  gamma (Sec. 2.4), relaxation (Eq. LBGK), A-A write.
 #pragma once
 
+#include <type_traits>
+
 #include "lbm_device.cuh"
 
 namespace lbm {
@@ -99,8 +101,9 @@ template <int D, int P, typename S, typename R, typename A>
 __global__ void __launch_bounds__(Blocks<D, R>::bx * Blocks<D, R>::by * Blocks<D, R>::bz,
                                   D == 3 && sizeof(R) == 4 ? LBM_K1_MINBLOCKS_F32 : 1)
 moments_eos_kernel(DevDomain d) {
-  moments_eos_node<D, P, S, R, A>(d, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y,
-                                  blockIdx.z * blockDim.z + threadIdx.z);
+  using B = Blocks<D, R>;
+  moments_eos_node<D, P, S, R, A>(d, blockIdx.x * B::bx + threadIdx.x, tile_y<D>() * B::by + threadIdx.y,
+                                  D == 3 ? blockIdx.z * B::bz + threadIdx.z : 0);
 }
 
 }  // namespace lbm
@@ -243,66 +246,6 @@ __device__ __forceinline__ void aux_force(const DevDomain& d, int x, int y, int 
 }
 
 // ---------------------------------------------------------------------------
-// Density and exact-difference-method velocity u + F/(2 rho); the auxiliary
-// fields must describe the current state (pass 1 run just before).
-// ---------------------------------------------------------------------------
-template <int D, typename S, typename R, typename A>
-__global__ void macroscopic_kernel(DevDomain d, int parity, double* rho_out, double* u_out) {
-  constexpr int Q = Lattice<D>::Q;
-  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= d.N) return;
-  const int x = (int)(n % d.nx), y = (int)((n / d.nx) % d.ny), z = (int)(n / ((long long)d.nx * d.ny));
-  R f[Q];
-  gather<D, S, R>(d, parity, x, y, z, f);
-  R rho, j[3], Pi[6];
-  moments<D, R>(f, rho, j, Pi);
-  R F[3];
-  aux_force<D, R, A>(d, x, y, z, rho, F);
-  rho_out[n] = (double)rho;
-  for (int a = 0; a < D; ++a) u_out[a * d.N + n] = (double)((j[a] + (R)0.5 * F[a]) / rho);
-}
-
-// ---------------------------------------------------------------------------
-// Largest speed |u + F/(2 rho)| of the reported velocity (the velocity
-// macroscopic_kernel writes), one partial maximum per block in field 4 of the
-// [block][5] layout that diag_final_kernel reduces (fields 0-3 zero).  The
-// auxiliary fields must describe the current state.
-// ---------------------------------------------------------------------------
-template <int D, typename S, typename R, typename A>
-__global__ void __launch_bounds__(256) max_speed_partial_kernel(DevDomain d, int parity, double* partial) {
-  constexpr int Q = Lattice<D>::Q;
-  __shared__ double sh[256];
-  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  double um = 0;
-  if (n < d.N) {
-    const int x = (int)(n % d.nx), y = (int)((n / d.nx) % d.ny), z = (int)(n / ((long long)d.nx * d.ny));
-    R f[Q];
-    gather<D, S, R>(d, parity, x, y, z, f);
-    R rho, j[3], Pi[6];
-    moments<D, R>(f, rho, j, Pi);
-    R F[3];
-    aux_force<D, R, A>(d, x, y, z, rho, F);
-    double u2 = 0;
-    for (int a = 0; a < D; ++a) {
-      const double ua = (double)((j[a] + (R)0.5 * F[a]) / rho);
-      u2 += ua * ua;
-    }
-    um = sqrt(u2);
-    if (!(um == um)) um = INFINITY;  // a non-finite state reports an infinite speed
-  }
-  sh[threadIdx.x] = um;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + s]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < 4; ++k) partial[blockIdx.x * 5 + k] = 0.0;
-    partial[blockIdx.x * 5 + 4] = sh[0];
-  }
-}
-
-// ---------------------------------------------------------------------------
 // Drop-on-film initial fields (float64, natural layout): see lbm_init_drop_on_film.
 // The white noise draws from SplitMix64 (Steele, Lea & Flood 2014) keyed by
 // (seed, node, component), two uniforms per value, normal by Box-Muller.
@@ -346,47 +289,57 @@ __global__ void drop_on_film_kernel(DevDomain d, double R, double film, double g
 
 // ---------------------------------------------------------------------------
 // Largest |grad rho| of the auxiliary density (second-order central differences;
-// the ghost layer supplies the wrapped or mirrored neighbours), one partial
-// maximum per block in field 4 of the diag layout.
+// the ghost layer supplies the wrapped or mirrored neighbours): kDiagBlocks blocks at
+// most, each over every gridDim-th tile of 32 x 8 nodes, one partial maximum per block.
+// Float64 is 58 times slower than float32, so a warp differences in float64 only the
+// nodes whose float32 gradient is not clearly below the largest it has met.
 // ---------------------------------------------------------------------------
+constexpr int kDiagBlocks = 152 * 6;
+
 template <int D, typename A>
-__global__ void __launch_bounds__(256) grad_partial_kernel(DevDomain d, double* partial) {
-  __shared__ double sh[256];
-  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  double gm = 0;
-  if (n < d.N) {
-    const int x = (int)(n % d.nx), y = (int)((n / d.nx) % d.ny), z = (int)(n / ((long long)d.nx * d.ny));
-    const Two<A>* a2 = (const Two<A>*)d.aux;
-    const long long pc = pnode_of<D>(d, x, y, z);
-    const long long e[3] = {1, d.px, (long long)d.px * d.py};
-    double g2 = 0;
-    for (int a = 0; a < D; ++a) {
-      const double ga = 0.5 * ((double)a2[pc + e[a]].x - (double)a2[pc - e[a]].x);
-      g2 += ga * ga;
+__global__ void __launch_bounds__(256) grad_partial_kernel(DevDomain d, int ntx, int nty, int ntiles, double* partial) {
+  const Two<A>* a2 = (const Two<A>*)d.aux;
+  const long long e[3] = {1, d.px, (long long)d.px * d.py};
+  float top = 0.0f;
+  double best = 0;
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int x = (t % ntx) * 32 + threadIdx.x, y = ((t / ntx) % nty) * 8 + threadIdx.y, z = t / (ntx * nty);
+    const bool in = x < d.nx && y < d.ny;
+    A r[2 * D];
+    float g2f = 0.0f;
+    if (in) {
+      const long long pc = pnode_of<D>(d, x, y, z);
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        r[2 * a] = a2[bc_pnode(d, pc - e[a])].x;
+        r[2 * a + 1] = a2[bc_pnode(d, pc + e[a])].x;
+        const float g = (float)(r[2 * a + 1] - r[2 * a]);
+        g2f = fmaf(g, g, g2f);
+      }
     }
-    gm = sqrt(g2);
+    // non-negative floats order as their bits; a NaN is above them all
+    top = fmaxf(top, __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(g2f))));
+    if (in && !(g2f < 0.99f * top)) {
+      double g2 = 0;
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        const double ga = 0.5 * ((double)r[2 * a + 1] - (double)r[2 * a]);
+        g2 += ga * ga;
+      }
+      best = fmax(best, g2);  // a NaN is passed over
+    }
   }
-  sh[threadIdx.x] = gm;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + s]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < 4; ++k) partial[blockIdx.x * 5 + k] = 0.0;
-    partial[blockIdx.x * 5 + 4] = sh[0];
-  }
+  block_max_store<256>(threadIdx.x + 32 * threadIdx.y, sqrt(best), partial, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
 // Crown radius: over the nodes of one layer (index `layer` along the last axis),
 // the largest distance from the vertical axis through the domain centre of a
-// node whose auxiliary density exceeds rho_mid; one partial maximum per block in
-// field 4 of the diag layout (0 where no node qualifies).
+// node whose auxiliary density exceeds rho_mid; one partial maximum per block
+// (0 where no node qualifies).
 // ---------------------------------------------------------------------------
 template <int D, typename A>
 __global__ void __launch_bounds__(256) crown_partial_kernel(DevDomain d, int layer, double rho_mid, double* partial) {
-  __shared__ double sh[256];
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long nl = D == 3 ? (long long)d.nx * d.ny : d.nx;
   double rm = 0;
@@ -400,16 +353,7 @@ __global__ void __launch_bounds__(256) crown_partial_kernel(DevDomain d, int lay
       rm = sqrt(dx * dx + dy * dy);
     }
   }
-  sh[threadIdx.x] = rm;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + s]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    for (int q = 0; q < 4; ++q) partial[blockIdx.x * 5 + q] = 0.0;
-    partial[blockIdx.x * 5 + 4] = sh[0];
-  }
+  block_max_store<256>(threadIdx.x, rm, partial, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -428,46 +372,121 @@ __global__ void bare_velocity_kernel(DevDomain d, const double* rho_in, double* 
 }
 
 // ---------------------------------------------------------------------------
-// Deterministic totals: per-block partial sums (fixed order), then one block.
+// Deterministic totals: kDiagBlocks blocks, each over every kDiagBlocks-th tile of
+// 32 x 8 nodes, then one block (diag_final_kernel) over their sums in a fixed order.
 // partial layout: [block][5] = mass, jx, jy, jz, max|u|.
+//
+// Bound by the float64 pipe.  The totals are linear in the populations, so a thread sums
+// each of its Q slots over all of its nodes (one addition per population) and forms the moments once at the end; max|u| needs the moments of every
+// node, which float32 storage forms in float32 first and in float64 only where the speed
+// is not clearly below the largest this thread has seen.
 // ---------------------------------------------------------------------------
-template <int D, typename S>
-__global__ void __launch_bounds__(256) diag_partial_kernel(DevDomain d, int parity, double* partial) {
-  constexpr int Q = Lattice<D>::Q;
-  __shared__ double sh[5][256];
-  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  double m = 0, jj[3] = {0, 0, 0}, um = 0;
-  if (n < d.N) {
-    const int x = (int)(n % d.nx), y = (int)((n / d.nx) % d.ny), z = (int)(n / ((long long)d.nx * d.ny));
-    double f[Q];
-    gather<D, S, double>(d, parity, x, y, z, f);
-    double Pi[6];
-    moments<D, double>(f, m, jj, Pi);
-    const double u2 = (jj[0] * jj[0] + jj[1] * jj[1] + jj[2] * jj[2]) / (m * m);
-    um = sqrt(u2);
-  }
-  sh[0][threadIdx.x] = m; sh[1][threadIdx.x] = jj[0]; sh[2][threadIdx.x] = jj[1];
-  sh[3][threadIdx.x] = jj[2]; sh[4][threadIdx.x] = um;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) {
-      for (int k = 0; k < 4; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + s];
-      sh[4][threadIdx.x] = fmax(sh[4][threadIdx.x], sh[4][threadIdx.x + s]);
+
+// g = (double)f, exactly.  For float32 by moving the fields of the bits where all Q values
+// are normal numbers: the float64 pipe, which also runs the conversion instruction, sets
+// the pace.
+template <int Q>
+__device__ __forceinline__ void widen(const float (&f)[Q], double (&g)[Q]) {
+  bool normal = true;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) normal = normal && (__float_as_uint(f[i]) & 0x7fffffffu) - 0x00800000u < 0x7f000000u;
+  if (normal) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const unsigned b = __float_as_uint(f[i]);
+      g[i] = __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
     }
-    __syncthreads();
+  } else {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) g[i] = (double)f[i];
   }
-  if (threadIdx.x == 0)
-    for (int k = 0; k < 5; ++k) partial[blockIdx.x * 5 + k] = sh[k][0];
+}
+template <int Q>
+__device__ __forceinline__ void widen(const double (&f)[Q], double (&g)[Q]) {
+#pragma unroll
+  for (int i = 0; i < Q; ++i) g[i] = f[i];
 }
 
-static __global__ void diag_final_kernel(const double* partial, int nblocks, double* out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double acc[5] = {0, 0, 0, 0, 0};
-  for (int b = 0; b < nblocks; ++b) {
-    for (int k = 0; k < 4; ++k) acc[k] += partial[b * 5 + k];
-    acc[4] = fmax(acc[4], partial[b * 5 + 4]);
+template <int D, typename S>
+__global__ void __launch_bounds__(256, 2) diag_partial_kernel(DevDomain d, int parity, int ntx, int nty, int ntiles,
+                                                              double* partial) {
+  constexpr int Q = Lattice<D>::Q;
+  using L = typename std::conditional<sizeof(S) == 4, float, double>::type;  // populations as loaded
+  __shared__ double sh[5][8];
+  const int tid = threadIdx.x + 32 * threadIdx.y;
+  double acc[Q], u2max = 0;
+  float top = 0.0f;  // largest float32 speed squared this warp has met
+#pragma unroll
+  for (int i = 0; i < Q; ++i) acc[i] = 0;
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int x = (t % ntx) * 32 + threadIdx.x, y = ((t / ntx) % nty) * 8 + threadIdx.y, z = t / (ntx * nty);
+    bool in = x < d.nx && y < d.ny;
+    L f[Q];
+    double g[Q];
+    float u2f = 0.0f;
+    if (in) {
+      gather<D, S, L>(d, parity, x, y, z, f);
+      if constexpr (sizeof(L) == 4) {
+        NodeMoments<float> m;
+        row_moments<D, float>(f, m);
+        u2f = (m.jx * m.jx + m.jy * m.jy + m.jz * m.jz) / (m.rho * m.rho);
+      }
+      widen<Q>(f, g);
+#pragma unroll
+      for (int i = 0; i < Q; ++i) acc[i] += g[i];
+    }
+    if constexpr (sizeof(L) == 4) {
+      // non-negative floats order as their bits; a NaN is above them all
+      top = fmaxf(top, __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(u2f))));
+      in = in && !(u2f < 0.999f * top);
+    }
+    if (in) {
+      NodeMoments<double> m;
+      row_moments<D, double>(g, m);
+      const double u2 = (m.jx * m.jx + m.jy * m.jy + m.jz * m.jz) / (m.rho * m.rho);
+      u2max = fmax(u2max, u2);  // a NaN is passed over
+    }
   }
-  for (int k = 0; k < 5; ++k) out[k] = acc[k];
+  NodeMoments<double> m;
+  row_moments<D, double>(acc, m);
+  double v[5] = {m.rho, m.jx, m.jy, m.jz, sqrt(u2max)};
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double w = __shfl_xor_sync(0xffffffffu, v[k], o);
+      v[k] = k < 4 ? v[k] + w : fmax(v[k], w);
+    }
+    if (threadIdx.x == 0) sh[k][threadIdx.y] = v[k];
+  }
+  __syncthreads();
+  if (tid < 5) {
+    double s = sh[tid][0];
+    for (int w = 1; w < 8; ++w) s = tid < 4 ? s + sh[tid][w] : fmax(s, sh[tid][w]);
+    partial[blockIdx.x * 5 + tid] = s;
+  }
+}
+
+// Sums (fields 0-3) and maximum (field 4) of the partials by one block of 32 x 5 threads:
+// warp k takes field k, every lane every 32nd block.  (One thread over all of them, with
+// one partial per 256 nodes, took 7.9 ms on 8.4 million nodes.)
+static __global__ void diag_final_kernel(const double* partial, int nblocks, double* out) {
+  const int k = threadIdx.y;
+  double v = 0;
+  for (int b = threadIdx.x; b < nblocks; b += 32) v = k < 4 ? v + partial[b * 5 + k] : fmax(v, partial[b * 5 + k]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double w = __shfl_xor_sync(0xffffffffu, v, o);
+    v = k < 4 ? v + w : fmax(v, w);
+  }
+  if (threadIdx.x == 0) out[k] = v;
+}
+
+// Largest of n partial maxima, by one block of 1024 threads.
+static __global__ void __launch_bounds__(1024) max_final_kernel(const double* partial, long long n, double* out) {
+  double v = 0;
+  for (long long b = threadIdx.x; b < n; b += 1024) v = fmax(v, partial[b]);
+  block_max_store<1024>(threadIdx.x, v, out, 0);
 }
 
 }  // namespace lbm

@@ -27,20 +27,23 @@ struct Ops {
   // modulo the domain) into out[Q][ez][ey][ex]
   void (*canonical_window)(const DevDomain&, int parity, const int origin[3], const int extent[3], double* out,
                            cudaStream_t);
-  void (*macroscopic)(const DevDomain&, int parity, double* rho, double* u, cudaStream_t);
+  // rho[N] and the reported velocity u[D*N] (float64) from the current auxiliary fields
+  void (*macroscopic)(const DevDomain&, const TileMaps& maps, double* rho, double* u, cudaStream_t);
   // u[a*N + n] -= F_a/(2 rho[n]), F from the current auxiliary fields
   void (*bare_velocity)(const DevDomain&, const double* rho, double* u, cudaStream_t);
-  // returns the number of partial blocks written to partial (5 doubles each)
+  // totals: [block][5] partials of kDiagBlocks blocks at most; returns their number
   int (*diag_partial)(const DevDomain&, int parity, double* partial, cudaStream_t);
-  // the same layout, field 4 = largest |u + F/(2 rho)| of the block (auxiliary fields current)
-  int (*max_speed_partial)(const DevDomain&, int parity, double* partial, cudaStream_t);
+  // Block maxima, reduced by launch_max_final: each returns the number of blocks, and
+  // launches nothing when partial is null.  The auxiliary fields must be current.
+  // largest |u + F/(2 rho)| of the block
+  long long (*speed_partial)(const DevDomain&, const TileMaps& maps, double* partial, cudaStream_t);
   // drop-on-film initial fields into rho[N], u[D*N] (device, float64)
   void (*drop_on_film)(const DevDomain&, const lbm_drop_on_film& g, double rho_l, double rho_v, double* rho, double* u,
                        cudaStream_t);
-  // the same layout, field 4 = largest |grad rho| of the block (auxiliary fields current)
-  int (*grad_partial)(const DevDomain&, double* partial, cudaStream_t);
-  // the same layout, field 4 = crown radius of the block's nodes of one layer
-  int (*crown_partial)(const DevDomain&, int layer, double rho_mid, double* partial, cudaStream_t);
+  // largest |grad rho| of the block
+  long long (*grad_partial)(const DevDomain&, double* partial, cudaStream_t);
+  // crown radius of the block's nodes of one layer
+  long long (*crown_partial)(const DevDomain&, int layer, double rho_mid, double* partial, cudaStream_t);
 };
 
 // Defined in lbm_d2q9.cu and lbm_d3q27.cu.
@@ -216,7 +219,11 @@ inline bool make_tile_maps(TileMaps* m, const DevDomain& d, int D, size_t elem_b
   return true;
 }
 
-// Final fixed-order reduction of the diagnostic partial sums (lbm_d2q9.cu).
+// Blocks of diag_partial.
+int diag_blocks();
+// Final fixed-order reductions (lbm_d2q9.cu): out[5] of the totals' partials, out[0] the
+// largest of n block maxima.
 void launch_diag_final(const double* partial, int nblocks, double* out, cudaStream_t s);
+void launch_max_final(const double* partial, long long n, double* out, cudaStream_t s);
 
 }  // namespace lbm
