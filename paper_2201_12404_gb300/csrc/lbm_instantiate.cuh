@@ -7,6 +7,19 @@
 
 namespace lbm {
 
+// Once per device, outside any capture: the dynamic shared memory limit of kernel K.
+template <auto K>
+inline void configure(size_t smem) {
+  constexpr int kMaxDev = 64;
+  static bool done[kMaxDev] = {};
+  if (smem <= 48 * 1024) return;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 0 && dev < kMaxDev && done[dev]) return;
+  cudaFuncSetAttribute((const void*)K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (dev >= 0 && dev < kMaxDev) done[dev] = true;
+}
+
 template <int D, typename S, typename R, typename A>
 struct Launch {
   using B = Blocks<D, R>;
@@ -20,43 +33,43 @@ struct Launch {
     }
     return dim3(gx, ty, (d.nz + B::bz - 1) / B::bz);
   }
-  static void moments_eos(const DevDomain& d, int parity, cudaStream_t s) {
-    if (parity == 0) moments_eos_kernel<D, 0, S, R, A><<<tile_grid(d), block(), 0, s>>>(d);
-    else moments_eos_kernel<D, 1, S, R, A><<<tile_grid(d), block(), 0, s>>>(d);
+  template <int P>
+  static void moments_eos_parity(const DevDomain& d, cudaStream_t s) {
+    constexpr auto k = moments_eos_kernel<D, P, S, R, A>;
+    k<<<tile_grid(d), block(), 0, s>>>(d);
   }
-  using QT = QTile<D, 2 * sizeof(A)>;
-  static dim3 qflux_grid(const DevDomain& d) {
-    return dim3((d.nx + QT::EX - 1) / QT::EX, (d.ny + QT::EY - 1) / QT::EY, (d.nz + QT::EZ - 1) / QT::EZ);
+  static void moments_eos(const DevDomain& d, int parity, cudaStream_t s) {
+    if (parity == 0) moments_eos_parity<0>(d, s);
+    else moments_eos_parity<1>(d, s);
+  }
+  template <bool kSmall> using QT = QTile<D, 2 * sizeof(A), kSmall>;
+  template <int kMode, bool kSmall>
+  static void qflux_tiles(const DevDomain& d, const TileMaps& maps, double* out0, double* out1, cudaStream_t s) {
+    using T = QT<kSmall>;
+    constexpr size_t smem = qflux_dyn_smem<D, T, A>();
+    constexpr auto k = qflux_tile_kernel<D, R, A, T, kMode>;
+    configure<k>(smem);
+    const dim3 g((d.nx + T::EX - 1) / T::EX, (d.ny + T::EY - 1) / T::EY, (d.nz + T::EZ - 1) / T::EZ);
+    k<<<g, dim3(T::TX, T::TY), smem, s>>>(d, maps, out0, out1);
   }
   template <int kMode>
   static void qflux_launch(const DevDomain& d, const TileMaps& maps, double* out0, double* out1, cudaStream_t s) {
-    constexpr size_t smem = qflux_dyn_smem<D, A>();
-    auto k = qflux_tile_kernel<D, R, A, kMode>;
-    constexpr int kMaxDev = 64;
-    static bool opted_in[kMaxDev] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (smem > 48 * 1024 && (dev < 0 || dev >= kMaxDev || !opted_in[dev])) {
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (dev >= 0 && dev < kMaxDev) opted_in[dev] = true;
-    }
-    k<<<qflux_grid(d), dim3(QT::TX, QT::TY), smem, s>>>(d, maps, out0, out1);
+    if (maps.qtile_small) qflux_tiles<kMode, true>(d, maps, out0, out1, s);
+    else qflux_tiles<kMode, false>(d, maps, out0, out1, s);
   }
   static void qflux(const DevDomain& d, const TileMaps& maps, cudaStream_t s) {
     qflux_launch<kQfluxStep>(d, maps, nullptr, nullptr, s);
   }
-  static void collide_stream(const DevDomain& d, const TileMaps& maps, int parity, cudaStream_t s) {
+  template <int P>
+  static void collide_stream_parity(const DevDomain& d, const TileMaps& maps, cudaStream_t s) {
     constexpr size_t smem = collide_dyn_smem<D, R>(B::bx * B::by * B::bz);
-    auto k = parity == 0 ? collide_stream_kernel<D, 0, S, R, A> : collide_stream_kernel<D, 1, S, R, A>;
-    constexpr int kMaxDev = 64;
-    static bool opted_in[2][kMaxDev] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= kMaxDev || !opted_in[parity][dev]) {
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (dev >= 0 && dev < kMaxDev) opted_in[parity][dev] = true;
-    }
+    constexpr auto k = collide_stream_kernel<D, P, S, R, A>;
+    configure<k>(smem);
     k<<<tile_grid(d), block(), smem, s>>>(d, maps);
+  }
+  static void collide_stream(const DevDomain& d, const TileMaps& maps, int parity, cudaStream_t s) {
+    if (parity == 0) collide_stream_parity<0>(d, maps, s);
+    else collide_stream_parity<1>(d, maps, s);
   }
   static unsigned blocks1d(const DevDomain& d) { return (unsigned)((d.N + 255) / 256); }
   static void init_equilibrium(const DevDomain& d, const double* rho, const double* ux, const double* uy,
@@ -98,9 +111,8 @@ struct Launch {
     return t.blocks;
   }
   static long long speed_partial(const DevDomain& d, const TileMaps& maps, double* partial, cudaStream_t s) {
-    const dim3 g = qflux_grid(d);
     if (partial) qflux_launch<kQfluxSpeed>(d, maps, partial, nullptr, s);
-    return (long long)g.x * g.y * g.z;
+    return maps.qtile_small ? tiles_of<QT<true>>(d) : tiles_of<QT<false>>(d);
   }
   static void drop_on_film(const DevDomain& d, const lbm_drop_on_film& g, double rho_l, double rho_v, double* rho,
                            double* u, cudaStream_t s) {

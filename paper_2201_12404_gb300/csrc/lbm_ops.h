@@ -130,10 +130,10 @@ inline bool make_aux_map(CUtensorMap* map, const DevDomain& d, int D, size_t ele
   return true;
 }
 
-// Tensor map over the q_a planes (element offset 2 PN of d.aux, one plane per
-// axis): a (px, py[, pz], D) tensor with a box of `tile` values of one plane.
-inline bool make_q_map(CUtensorMap* map, const DevDomain& d, int D, size_t elem_bytes, const cuuint32_t tile[3],
-                       const char** why) {
+// Tensor map over the D planes of d.aux from plane `first` on (2: q_a, 2 + D: j_a, then
+// F_a): a (px, py[, pz], D) tensor with a box of `tile` values of one plane.
+inline bool make_plane_map(CUtensorMap* map, const DevDomain& d, int D, size_t elem_bytes, int first,
+                           const cuuint32_t tile[3], const char** why) {
   const tensor_map_encode_fn encode = tensor_map_encoder(why);
   if (!encode) return false;
   const cuuint64_t e = elem_bytes;
@@ -154,12 +154,12 @@ inline bool make_q_map(CUtensorMap* map, const DevDomain& d, int D, size_t elem_
     strides[1] = (cuuint64_t)d.PN * e;
     box[2] = 1;
   }
-  void* base = (char*)d.aux + 2 * (size_t)d.PN * elem_bytes;
+  void* base = (char*)d.aux + first * (size_t)d.PN * elem_bytes;
   const CUresult r = encode(map, elem_bytes == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
                             rank, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
-    *why = "cuTensorMapEncodeTiled rejected the q tensor map";
+    *why = "cuTensorMapEncodeTiled rejected a plane tensor map";
     return false;
   }
   return true;
@@ -184,11 +184,31 @@ inline void fill_geometry(DevDomain& d, const lbm_params& p, int D, size_t pop_b
   fill_slot_offsets(d, D, pop_bytes);
 }
 
-// The halo box of QTile<D, pair bytes> for pass 1b.
+// Which tile pass 1b takes.  2-D and float64: the small one where the large ones would
+// not fill the SMs once (128x128 2-D float32, passes 1 + 1b: 11.4 us small, 13.5 large;
+// the 800x10 column in float64 14.5 and 27 us).  3-D float32: the small one, 25 KB of
+// shared memory a block against 34, up to 160 large tiles per SM (19 million nodes).
+// Alone the large one gains there too (512x512x256: 2.10 ms against 2.14; 203x187x149:
+// 220 us against 221; 67x67x67: 32.0 against 30.3), but six large blocks take nearly all of
+// an SM's shared memory, and beside the other kernels of domains on other streams the SM
+// divides its memory anew for them: four cubes of 64 to 128 took 460 us a step against 380.
+template <typename T>
+inline long long tiles_of(const DevDomain& d) {
+  return (long long)((d.nx + T::EX - 1) / T::EX) * ((d.ny + T::EY - 1) / T::EY) * ((d.nz + T::EZ - 1) / T::EZ);
+}
 template <int D, int kPairBytes>
-inline void qtile_box(cuuint32_t box[3]) {
-  using T = QTile<D, kPairBytes>;
-  box[0] = T::HX; box[1] = T::HY; box[2] = T::HZ;
+inline bool qtile_small(const DevDomain& d) {
+  return tiles_of<QTile<D, kPairBytes, false>>(d) < 152 * (D == 2 ? 3 : (kPairBytes == 8 ? 160 : 6));
+}
+
+// The halo box of QTile for pass 1b.
+template <int D, int kPairBytes>
+inline void qtile_box(cuuint32_t box[3], bool small) {
+  using T = QTile<D, kPairBytes, false>;
+  using U = QTile<D, kPairBytes, true>;
+  box[0] = small ? U::HX : T::HX;
+  box[1] = small ? U::HY : T::HY;
+  box[2] = small ? U::HZ : T::HZ;
 }
 
 // The q box of axis a for a tile of pass 2.
@@ -203,18 +223,25 @@ inline bool make_tile_maps(TileMaps* m, const DevDomain& d, int D, size_t elem_b
   // pass 1b: a QTile tile with a 2-node halo
   cuuint32_t box[3];
   if (D == 3) {
-    if (elem_bytes == 4) qtile_box<3, 8>(box); else qtile_box<3, 16>(box);
+    m->qtile_small = elem_bytes == 4 ? qtile_small<3, 8>(d) : qtile_small<3, 16>(d);
+    if (elem_bytes == 4) qtile_box<3, 8>(box, m->qtile_small); else qtile_box<3, 16>(box, m->qtile_small);
   } else {
-    if (elem_bytes == 4) qtile_box<2, 8>(box); else qtile_box<2, 16>(box);
+    m->qtile_small = elem_bytes == 4 ? qtile_small<2, 8>(d) : qtile_small<2, 16>(d);
+    if (elem_bytes == 4) qtile_box<2, 8>(box, m->qtile_small); else qtile_box<2, 16>(box, m->qtile_small);
   }
   if (!make_aux_map(&m->aux_q, d, D, elem_bytes, box, why)) return false;
+  if (D == 3) {  // the tile without its halo, the full width in x
+    box[1] -= 4;
+    box[2] -= 4;
+    if (!make_plane_map(&m->j, d, D, elem_bytes, 2 + D, box, why)) return false;
+  }
   for (int a = 0; a < D; ++a) {
     if (D == 3) {
       if (elem_bytes == 4) qbox_tile<3, float>(a, box); else qbox_tile<3, double>(a, box);
     } else {
       if (elem_bytes == 4) qbox_tile<2, float>(a, box); else qbox_tile<2, double>(a, box);
     }
-    if (!make_q_map(&m->q[a], d, D, elem_bytes, box, why)) return false;
+    if (!make_plane_map(&m->q[a], d, D, elem_bytes, 2, box, why)) return false;
   }
   return true;
 }
