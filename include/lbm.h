@@ -148,8 +148,8 @@ lbm_status lbm_init_fields(lbm_handle h, const double* rho, const double* ux, co
  * kernels: moments and the Peng-Robinson pseudo-potential (Sec. 2.3); the force
  * of Eq. (Kforce_final) and the flux q of Eq. (correction); the collision of
  * Sec. 2.4 with the A-A stream.  With timing off, once the domain has run two
- * steps, pairs of steps are replayed as a captured CUDA graph of those kernels
- * (same kernels and arguments, bit-identical results; recaptured when the gamma
+ * steps, groups of eight and of two steps are replayed as captured CUDA graphs of those
+ * kernels (same kernels and arguments, bit-identical results; recaptured when the gamma
  * record is switched on).  An instability detected by an earlier call surfaces
  * here or in any later synchronising call as LBM_ERR_UNSTABLE. */
 lbm_status lbm_step(lbm_handle h, int64_t nsteps);

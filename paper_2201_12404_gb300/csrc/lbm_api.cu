@@ -247,25 +247,26 @@ lbm_status launch_k(lbm_domain* h, int kind) {
   return LBM_OK;
 }
 
-// Launch the graph of two steps from the current parity, capturing it first if
-// there is none for this parity and gamma record.  *replayed is false (and nothing
+// Launch the graph of kGraphSteps[kind] steps from the current parity, capturing it first
+// if there is none for this parity and gamma record.  *replayed is false (and nothing
 // was enqueued) when capture is not possible on this stream; the domain then keeps
 // to plain launches.
-lbm_status launch_pair_graph(lbm_domain* h, bool* replayed) {
+lbm_status launch_step_graph(lbm_domain* h, int kind, bool* replayed) {
   *replayed = false;
-  const int p = h->parity;
-  if (!h->step_graph[p] || h->step_graph_gamma[p] != h->dev.gamma_out) {
-    if (h->step_graph[p]) {
-      cudaGraphExecDestroy(h->step_graph[p]);
-      h->step_graph[p] = nullptr;
+  const int p = h->parity, steps = lbm_domain::kGraphSteps[kind];
+  lbm_domain::StepGraph& sg = h->step_graph[kind][p];
+  if (!sg.exec || sg.gamma != h->dev.gamma_out) {
+    if (sg.exec) {
+      cudaGraphExecDestroy(sg.exec);
+      sg.exec = nullptr;
     }
     if (cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
       cudaGetLastError();
       h->graphs_ok = false;
       return LBM_OK;
     }
-    for (int k = 0; k < 2; ++k) {
-      const int par = p ^ k;
+    for (int k = 0; k < steps; ++k) {
+      const int par = p ^ (k & 1);
       h->ops->moments_eos(h->dev, par, h->stream);
       h->ops->qflux(h->dev, h->maps, h->stream);
       h->ops->collide_stream(h->dev, h->maps, par, h->stream);
@@ -280,11 +281,11 @@ lbm_status launch_pair_graph(lbm_domain* h, bool* replayed) {
       h->graphs_ok = false;
       return LBM_OK;
     }
-    h->step_graph[p] = exec;
-    h->step_graph_gamma[p] = (float*)h->dev.gamma_out;
+    sg.exec = exec;
+    sg.gamma = (float*)h->dev.gamma_out;
   }
-  LBM_CUDA(h, cudaGraphLaunch(h->step_graph[p], h->stream));
-  h->launches += 6;
+  LBM_CUDA(h, cudaGraphLaunch(sg.exec, h->stream));
+  h->launches += 3 * steps;
   *replayed = true;
   return LBM_OK;
 }
@@ -514,8 +515,9 @@ lbm_status lbm_destroy(lbm_handle h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   for (auto& m : h->marks) { cudaEventDestroy(m.a); cudaEventDestroy(m.b); }
   for (auto e : h->ev_pool) cudaEventDestroy(e);
-  for (auto& g : h->step_graph)
-    if (g) cudaGraphExecDestroy(g);
+  for (auto& kind : h->step_graph)
+    for (auto& g : kind)
+      if (g.exec) cudaGraphExecDestroy(g.exec);
   keep_free(h->p, h->dev.f);
   keep_free(h->p, h->dev.aux);
   keep_free(h->p, h->dev.rho_w[0]);
@@ -598,11 +600,13 @@ lbm_status lbm_step(lbm_handle h, int64_t nsteps) {
   if (!h->record_gamma) h->dev.gamma_out = nullptr;
   for (int64_t s = 0; s < nsteps;) {
     if (!h->timing && h->graphs_ok && h->plain_steps >= 2 && nsteps - s >= 2) {
+      const int kind = nsteps - s >= lbm_domain::kGraphSteps[1] ? 1 : 0;
       bool replayed = false;
-      if ((st = launch_pair_graph(h, &replayed)) != LBM_OK) break;
+      if ((st = launch_step_graph(h, kind, &replayed)) != LBM_OK) break;
       if (replayed) {
-        h->steps += 2;  // two steps: the parity is back where it was
-        s += 2;
+        // an even number of steps: the parity is back where it was
+        h->steps += lbm_domain::kGraphSteps[kind];
+        s += lbm_domain::kGraphSteps[kind];
         continue;
       }
     }

@@ -35,12 +35,19 @@ struct lbm_domain {
   int64_t cnt[2] = {0, 0};
   bool record_gamma = false;
   bool gamma_recorded = false;  // a step has run with recording on since the buffer was made
-  // CUDA graphs of two consecutive steps starting at parity p (the three kernels of
-  // parity p, then of 1 - p), replayed by lbm_step when timing is off.  A graph holds
-  // the kernel arguments of its capture, so it is keyed by the only device pointer
-  // that changes after creation, the gamma record (nullptr while not recording).
-  cudaGraphExec_t step_graph[2] = {nullptr, nullptr};
-  float* step_graph_gamma[2] = {nullptr, nullptr};
+  // CUDA graphs of an even number of consecutive steps starting at parity p (the three
+  // kernels of parity p, then of 1 - p, ...), replayed by lbm_step when timing is off.  A
+  // graph holds the kernel arguments of its capture, so it is keyed by the only device
+  // pointer that changes after creation, the gamma record (nullptr while not recording).
+  // Eight steps a graph, and two for what is left of a call: the gap between two graph
+  // launches is longer than between kernels within one (128x128 2-D float32: 9.0 us a step
+  // in graphs of two steps, 7.6 in eight, 7.4 in thirty-two; 67x67x67: 42.8, 41.4, 41.4).
+  static constexpr int kGraphSteps[2] = {2, 8};
+  struct StepGraph {
+    cudaGraphExec_t exec = nullptr;
+    float* gamma = nullptr;
+  };
+  StepGraph step_graph[2][2];  // [kind of kGraphSteps][parity]
   bool graphs_ok = true;   // cleared if capture or instantiation fails: plain launches then
   int64_t plain_steps = 0; // steps launched one kernel at a time (the launchers set their
                            // kernel attributes on first use, outside any capture)
