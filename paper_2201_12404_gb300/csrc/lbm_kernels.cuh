@@ -59,6 +59,10 @@ __device__ __forceinline__ void moments_eos_node(const DevDomain& d, int x, int 
   a2[pn] = pair;
 #pragma unroll
   for (int a = 0; a < D; ++a) aux[(2 + D + a) * d.PN + pn] = (A)j[a];
+  // a ghost images only nodes within one of a face
+  if ((unsigned)(x - 2) < (unsigned)(d.nx - 4) && (unsigned)(y - 2) < (unsigned)(d.ny - 4) &&
+      (D == 2 || (unsigned)(z - 2) < (unsigned)(d.nz - 4)))
+    return;
   bool wall = false;
   const int gx = ghost_of(x, d.nx, d.wall_lo[0], d.wall_hi[0], &wall);
   const int gy = ghost_of(y, d.ny, d.wall_lo[1], d.wall_hi[1], &wall);

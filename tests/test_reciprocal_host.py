@@ -1,4 +1,4 @@
-"""The float32 reciprocal and quotient of the collision kernel (one Newton-Raphson
+"""The float32 reciprocal, quotient and square root of the kernels (one Newton-Raphson
 step with a fused residual from a hardware approximation), emulated with exact
 float64 products: within one ulp of the true value for any approximation that is
 itself within two ulps, over the magnitudes the kernels meet."""
@@ -20,7 +20,7 @@ def approx(x, off):
 
 
 @pytest.mark.parametrize("off", [-2, -1, 0, 1, 2])
-def test_reciprocal_and_quotient_within_an_ulp(off):
+def test_reciprocal_quotient_and_root_within_an_ulp(off):
     rng = np.random.default_rng(7)
     x = np.exp(rng.uniform(np.log(1e-6), np.log(1e6), 200000)).astype(F)
     r0 = approx(x, off)
@@ -33,3 +33,9 @@ def test_reciprocal_and_quotient_within_an_ulp(off):
     q = fma(fma(-q, x, a), r0, q)
     true = a.astype(np.float64) / x.astype(np.float64)
     assert (np.abs(q - true) <= np.spacing(np.abs(true).astype(F))).all()
+    y0 = (1.0 / np.sqrt(x.astype(np.float64))).astype(F)
+    y0 = (y0.astype(np.float64) + off * np.spacing(y0)).astype(F)
+    s = (x * y0).astype(F)
+    s = fma(fma(-s, s, x), (F(0.5) * y0).astype(F), s)
+    true = np.sqrt(x.astype(np.float64))
+    assert (np.abs(s - true) <= np.spacing(true.astype(F))).all()
