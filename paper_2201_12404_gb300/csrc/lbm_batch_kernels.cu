@@ -2,7 +2,7 @@
 // nsteps time steps in one launch.  The blocks of a cooperative launch walk the
 // work list of tiles (every job's interior) three times per step, for pass 1,
 // pass 1b and pass 2, with a grid barrier after each.  The per-tile work is the
-// same code as the single-domain kernels (moments_eos_node, qflux_tile_staged,
+// same code as the single-domain kernels (moments_eos_tile, qflux_tile_staged,
 // collide_tile), with pass 1b's halo tile staged by warps.
 #include "../../include/lbm.h"
 #include "lbm_batch.h"
@@ -62,9 +62,8 @@ __global__ void __launch_bounds__(BX * BY, sizeof(R) == 4 ? LBM_BATCH_MINBLOCKS_
     for (int it = blockIdx.x; it < a.n_k2; it += gridDim.x) {
       const BatchItem w = a.k2[it];
       const DevDomain& d = a.jobs[w.job];
-      const int x = w.tx * BX + threadIdx.x, y = w.ty * BY + threadIdx.y;
-      if (((a.parity[w.job] + s) & 1) == 0) moments_eos_node<2, 0, S, R, A>(d, x, y, 0);
-      else moments_eos_node<2, 1, S, R, A>(d, x, y, 0);
+      if (((a.parity[w.job] + s) & 1) == 0) moments_eos_tile<2, 0, S, R, A>(d, w.tx * BX, w.ty * BY, 0, BX, BY, 1);
+      else moments_eos_tile<2, 1, S, R, A>(d, w.tx * BX, w.ty * BY, 0, BX, BY, 1);
     }
     if (!grid_barrier(a.barrier, a.error, a.poll_limit, a.skip_arrival)) return;
     // pass 1b: q over the interior tiles (and the ghosts imaging them)

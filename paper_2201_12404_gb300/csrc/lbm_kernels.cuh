@@ -41,12 +41,12 @@ __device__ __forceinline__ int ghost_image(int cp, int n, int wlo, int whi, bool
 // their stencils without wrap logic; j goes to the node alone (pass 1b reads it
 // there).  A warp is one aligned x row of 32 interior nodes, so each of its 27
 // population loads is one 128-byte line.
-template <int D, int P, typename S, typename R, typename A>
+template <int D, int P, typename S, typename R, typename A, bool kFace>
 __device__ __forceinline__ void moments_eos_node(const DevDomain& d, int x, int y, int z) {
   constexpr int Q = Lattice<D>::Q;
   if (x >= d.nx || y >= d.ny || z >= d.nz) return;
   R f[Q];
-  gather<D, P, S, R>(d, x, y, z, f);
+  gather<D, P, S, R, kFace>(d, x, y, z, f);
   NodeMoments<R> m;
   row_moments<D, R>(f, m);
   const R rho = m.rho, j[3] = {m.jx, m.jy, m.jz};
@@ -76,6 +76,14 @@ __device__ __forceinline__ void moments_eos_node(const DevDomain& d, int x, int 
   }
 }
 
+// Pass 1 on the tile of EX x EY x EZ nodes at (x0, y0, z0), one per thread of the block.
+template <int D, int P, typename S, typename R, typename A>
+__device__ __forceinline__ void moments_eos_tile(const DevDomain& d, int x0, int y0, int z0, int EX, int EY, int EZ) {
+  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + (D == 3 ? threadIdx.z : 0);
+  if ((P == 1 || DevStorage<S>::value) && tile_on_face<D>(d, x0, y0, z0, EX, EY, EZ)) moments_eos_node<D, P, S, R, A, true>(d, x, y, z);
+  else moments_eos_node<D, P, S, R, A, false>(d, x, y, z);
+}
+
 // The (rho, psi) pairs of every padded node straight from a density field
 // (device, float64, N values), ghosts included: what pass 1 writes for a state
 // whose density is that field, without forming populations first.  q is left
@@ -95,19 +103,23 @@ __global__ void __launch_bounds__(256) aux_density_kernel(DevDomain d, const dou
   ((Two<A>*)d.aux)[pn] = two<A>((A)rho, (A)psi_of<R>(d, rho));
 }
 
-// Resident blocks per SM asked of the register allocator: 16 of 64 threads, 64
-// registers, in the D3Q27 float32 and float16 kernels (256x256x128 impact in float16
-// deviations, passes 1 + 1b: 351 us, 372 before, at 76 registers in odd steps).
+// Resident 64-thread blocks per SM asked of the register allocator in 3-D float32
+// arithmetic: 20 (48 registers) for float32 storage, passes 1 + 1b on the 203x187x149 impact
+// 215 us against 223 at 16 and 227 at 12; 16 (64) for float16 deviations, on 256x256x128
+// 319 us against 323 at 20 and 337 at 12.
 #ifndef LBM_K1_MINBLOCKS_F32
-#define LBM_K1_MINBLOCKS_F32 16
+#define LBM_K1_MINBLOCKS_F32 20
+#endif
+#ifndef LBM_K1_MINBLOCKS_F16
+#define LBM_K1_MINBLOCKS_F16 16
 #endif
 template <int D, int P, typename S, typename R, typename A>
 __global__ void __launch_bounds__(Blocks<D, R>::bx * Blocks<D, R>::by * Blocks<D, R>::bz,
-                                  D == 3 && sizeof(R) == 4 ? LBM_K1_MINBLOCKS_F32 : 1)
+                                  D == 3 && sizeof(R) == 4 ? (sizeof(S) == 2 ? LBM_K1_MINBLOCKS_F16 : LBM_K1_MINBLOCKS_F32) : 1)
 moments_eos_kernel(DevDomain d) {
   using B = Blocks<D, R>;
-  moments_eos_node<D, P, S, R, A>(d, blockIdx.x * B::bx + threadIdx.x, tile_y<D>() * B::by + threadIdx.y,
-                                  D == 3 ? blockIdx.z * B::bz + threadIdx.z : 0);
+  moments_eos_tile<D, P, S, R, A>(d, blockIdx.x * B::bx, tile_y<D>() * B::by, D == 3 ? blockIdx.z * B::bz : 0, B::bx, B::by,
+                                  B::bz);
 }
 
 }  // namespace lbm
@@ -139,12 +151,11 @@ __global__ void init_equilibrium_kernel(DevDomain d, const double* rho, const do
     // each slot is encoded against the density of its upstream (writer) node; the
     // next step (even parity) decodes with rho_w[0] of that node
     const int x = (int)(n % d.nx), y = (int)((n / d.nx) % d.ny), z = (int)(n / ((long long)d.nx * d.ny));
-    const bool fast = fast_links<D>(d, x, y, z);
-    const XBase xb = xbase<S>(d, x, n);
+    const FaceLinks<D> fl(d, x, y, z);
     d.rho_w[0][n] = (float)r;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      const R rw = (R)(float)rho[upstream_node<D>(d, fast, xb, x, y, z, n, i)];
+      const R rw = (R)(float)rho[upstream_node<D>(d, fl, n, i)];
       const R feq = r * X[0][cxi(i) + 1] * X[1][cyi(i) + 1] * X[2][D == 3 ? czi(i) + 1 : 1];
       F[(long long)i * d.N + n] = __float2half_rn((float)(feq / ((R)wq<D>(i) * rw) - (R)1));
     }
@@ -198,10 +209,9 @@ __global__ void canonical_write_kernel(DevDomain d, const double* in) {
   if constexpr (DevStorage<S>::value) {
     // rho_w[0] holds every node's density (canonical_density_kernel, launched before)
     const int x = (int)(n % d.nx), y = (int)((n / d.nx) % d.ny), z = (int)(n / ((long long)d.nx * d.ny));
-    const bool fast = fast_links<D>(d, x, y, z);
-    const XBase xb = xbase<S>(d, x, n);
+    const FaceLinks<D> fl(d, x, y, z);
     for (int i = 0; i < Q; ++i) {
-      const double rw = (double)d.rho_w[0][upstream_node<D>(d, fast, xb, x, y, z, n, i)];
+      const double rw = (double)d.rho_w[0][upstream_node<D>(d, fl, n, i)];
       F[(long long)i * d.N + n] = __float2half_rn((float)(in[(long long)i * d.N + n] / (wq<D>(i) * rw) - 1.0));
     }
   } else {
