@@ -104,7 +104,21 @@ inline void fill_phys(DevDomain& d, const lbm_params& p, int D) {
   for (int k = 0; k < 3; ++k) pf.sgn_t[k] = float_at_or_above(pd.sgn_t[k]);
   pf.sgn0 = (float)pd.sgn0;
   d.gamma_mode = p.gamma_mode;
-  d.eos_fp64 = p.eos_fp64;
+  // rho |N| / M = |P - rho/3|: with t = b rho, N = 3 RT (1 + 2t - t^2) - 3 aalpha rho (1 - t) - M/3
+  // and M = 3 (1 - t)(1 + 2t - t^2).
+  const double num[4] = {3 * e.RT - 1, (6 * e.RT - 1) * e.b - 3 * e.aalpha, ((3 - 3 * e.RT) * e.b + 3 * e.aalpha) * e.b,
+                         -e.b * e.b * e.b};
+  const double den[4] = {3, 3 * e.b, -9 * e.b * e.b, 3 * e.b * e.b * e.b};
+  for (int k = 0; k < 4; ++k) {
+    d.eos_num[k].x = (float)num[k]; d.eos_num[k].y = (float)(num[k] - d.eos_num[k].x);
+    d.eos_den[k].x = (float)den[k]; d.eos_den[k].y = (float)(den[k] - d.eos_den[k].x);
+  }
+  // The pairs need the poles outside the band and products well inside float32's range;
+  // every calibrated parameter set of the equation is (b rho < 1, the rest of order one).
+  auto moderate = [](double x) { return std::fabs(x) > 1e-6 && std::fabs(x) < 1e6; };
+  const bool pairs = e.b * p.rho_liquid < 1 && moderate(e.b) && moderate(e.RT) && moderate(e.aalpha) &&
+                     moderate(p.rho_liquid) && p.rho_vapour > 0;
+  d.eos = p.eos_fp64 == 1 && !pairs ? kEosBandFloat64 : p.eos_fp64;
 }
 
 }  // namespace lbm
