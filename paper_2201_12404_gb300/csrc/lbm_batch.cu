@@ -16,7 +16,7 @@
 #include "lbm_handle.h"
 
 using lbm::BatchArgs;
-using lbm::BatchItem;
+using lbm::BatchTiles;
 using lbm::BatchVariant;
 using lbm::DevDomain;
 
@@ -30,9 +30,9 @@ struct lbm_batch {
   // device buffers
   DevDomain* d_jobs = nullptr;
   int* d_parity = nullptr;
-  BatchItem* d_items = nullptr;  // the tiles of every job's interior
+  BatchTiles* d_tiles = nullptr;  // the tiles of every job's interior
   unsigned int* d_sync = nullptr;  // [0] arrivals, [1] generation, [2] error word
-  int n_k2 = 0, grid = 0;
+  int ntiles = 0, grid = 0;
   std::map<int64_t, cudaGraphExec_t> graphs;
   bool use_graph = true;
   unsigned int poll_limit = lbm::kBarrierPollsDefault;
@@ -62,31 +62,33 @@ lbm_status bfail(lbm_batch* b, lbm_status st, const std::string& msg) {
 
 // Work list of a tile shape: the tiles of every job's interior (each pass walks
 // them; pass 1 writes the ghost images of its nodes itself).
-void build_items(const std::vector<lbm_domain*>& doms, int bx, int by, std::vector<BatchItem>& k2) {
-  k2.clear();
-  for (int j = 0; j < (int)doms.size(); ++j) {
-    const DevDomain& d = doms[j]->dev;
-    for (int ty = 0; ty < (d.ny + by - 1) / by; ++ty)
-      for (int tx = 0; tx < (d.nx + bx - 1) / bx; ++tx) k2.push_back({j, tx, ty});
+std::vector<BatchTiles> build_tiles(const std::vector<lbm_domain*>& doms, int bx, int by) {
+  std::vector<BatchTiles> tiles;
+  int first = 0;
+  for (const lbm_domain* h : doms) {
+    const int ntx = (h->dev.nx + bx - 1) / bx, nty = (h->dev.ny + by - 1) / by;
+    tiles.push_back({first, ntx});
+    first += ntx * nty;
   }
+  tiles.push_back({first, 1});
+  return tiles;
 }
 
-// Upload the work lists of variant v and size the cooperative grid.
+// Upload the work list of variant v and size the cooperative grid.
 lbm_status select_variant(lbm_batch* b, int v) {
   const BatchVariant& var = b->variants[v];
-  std::vector<BatchItem> k2;
-  build_items(b->doms, var.bx, var.by, k2);
-  if (b->d_items) { cudaFree(b->d_items); b->d_items = nullptr; }
-  B_CUDA(b, cudaMalloc(&b->d_items, k2.size() * sizeof(BatchItem)));
-  B_CUDA(b, cudaMemcpy(b->d_items, k2.data(), k2.size() * sizeof(BatchItem), cudaMemcpyHostToDevice));
-  b->n_k2 = (int)k2.size();
+  const std::vector<BatchTiles> tiles = build_tiles(b->doms, var.bx, var.by);
+  if (b->d_tiles) { cudaFree(b->d_tiles); b->d_tiles = nullptr; }
+  B_CUDA(b, cudaMalloc(&b->d_tiles, tiles.size() * sizeof(BatchTiles)));
+  B_CUDA(b, cudaMemcpy(b->d_tiles, tiles.data(), tiles.size() * sizeof(BatchTiles), cudaMemcpyHostToDevice));
+  b->ntiles = tiles.back().first;
   int dev = 0, sms = 0, per_sm = 0;
   B_CUDA(b, cudaGetDevice(&dev));
   B_CUDA(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   B_CUDA(b, cudaFuncSetAttribute(var.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)var.dyn_smem));
   B_CUDA(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, var.kernel, var.bx * var.by, var.dyn_smem));
   if (per_sm < 1) return bfail(b, LBM_ERR_CUDA, "the batch kernel cannot be resident on an SM");
-  b->grid = std::max(1, std::min(per_sm * sms, b->n_k2));
+  b->grid = std::max(1, std::min(per_sm * sms, b->ntiles));
   b->chosen = v;
   for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
   b->graphs.clear();
@@ -98,8 +100,8 @@ BatchArgs make_args(lbm_batch* b, const DevDomain* jobs, int* parity, int nsteps
   a.jobs = jobs;
   a.parity = parity;
   a.njobs = (int)b->doms.size();
-  a.k2 = b->d_items;
-  a.n_k2 = b->n_k2;
+  a.tiles = b->d_tiles;
+  a.ntiles = b->ntiles;
   a.barrier = b->d_sync;
   a.error = b->d_sync + 2;
   a.nsteps = nsteps;
@@ -174,7 +176,7 @@ lbm_status lbm_batch_destroy(lbm_batch_handle b) {
   for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
   if (b->d_jobs) cudaFree(b->d_jobs);
   if (b->d_parity) cudaFree(b->d_parity);
-  if (b->d_items) cudaFree(b->d_items);
+  if (b->d_tiles) cudaFree(b->d_tiles);
   if (b->d_sync) cudaFree(b->d_sync);
   delete b;
   return LBM_OK;

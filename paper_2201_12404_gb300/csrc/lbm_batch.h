@@ -8,17 +8,18 @@
 
 namespace lbm {
 
-// One tile of work: job index and tile coordinates in tile units.
-struct BatchItem {
-  int job, tx, ty;
+// The tiles of a job's interior in the work list: tile t of the list, first <= t < the
+// next job's first, is tile ((t - first) mod ntx, (t - first) / ntx) of the job.
+struct BatchTiles {
+  int first, ntx;
 };
 
 struct BatchArgs {
   const DevDomain* jobs;  // device array, one per job
   int* parity;            // device array: A-A parity of every job; flipped by the kernel at the end
   int njobs;
-  const BatchItem* k2;    // tiles over the interior of every job (all three passes)
-  int n_k2;
+  const BatchTiles* tiles;  // njobs + 1 entries, the last one's first = ntiles
+  int ntiles;
   unsigned int* barrier;  // [0] arrivals, [1] generation
   unsigned int* error;    // bit 1: a bounded grid-barrier wait gave up
   int nsteps;
