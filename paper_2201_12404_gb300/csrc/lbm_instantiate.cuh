@@ -33,8 +33,28 @@ struct Launch {
     }
     return dim3(gx, ty, (d.nz + B::bz - 1) / B::bz);
   }
+  // Whether passes 1 and 2 take consecutive nodes of a layer instead of tiles: where tiles
+  // would idle more than 8% of their lanes.  Without tiles pass 2 reads q from global
+  // memory, which costs more than it gives where few lanes idle (pass 2 of 512x512x256
+  // in float32: 2.69 ms against 2.58, of 128^3 90.0 us against 87.6) and less elsewhere
+  // (67^3, 46% idle: 16.4 us against 19.4; 107^3, 21%: 54.5, 57.5; 85^3, 14%: 26.6, 28.5;
+  // 203x187x149, 11%: 239.8, 239.5 and in float16 deviations 233, 255).  Pass 1 gains
+  // up to 2.5 us of 26 and never lost more than 1%.
+  static bool flat(const DevDomain& d) {
+    if (D == 2 || (long long)d.nx * d.ny >= 1 << 30 || d.nz > 65535) return false;
+    const long long lanes = (long long)((d.nx + B::bx - 1) / B::bx * B::bx) * ((d.ny + B::by - 1) / B::by * B::by);
+    return 100 * lanes > 108 * ((long long)d.nx * d.ny);
+  }
+  static dim3 flat_grid(const DevDomain& d) { return dim3((d.nx * d.ny + kFlatThreads - 1) / kFlatThreads, d.nz); }
   template <int P>
   static void moments_eos_parity(const DevDomain& d, cudaStream_t s) {
+    if constexpr (D == 3) {
+      if (flat(d)) {
+        constexpr auto k = moments_eos_flat_kernel<P, S, R, A>;
+        k<<<flat_grid(d), kFlatThreads, 0, s>>>(d);
+        return;
+      }
+    }
     constexpr auto k = moments_eos_kernel<D, P, S, R, A>;
     k<<<tile_grid(d), block(), 0, s>>>(d);
   }
@@ -62,6 +82,15 @@ struct Launch {
   }
   template <int P>
   static void collide_stream_parity(const DevDomain& d, const TileMaps& maps, cudaStream_t s) {
+    if constexpr (D == 3) {
+      if (flat(d)) {
+        constexpr size_t smem = collide_dyn_smem<D, R>(kFlatThreads);
+        constexpr auto k = collide_stream_flat_kernel<P, S, R, A>;
+        configure<k>(smem);
+        k<<<flat_grid(d), kFlatThreads, smem, s>>>(d);
+        return;
+      }
+    }
     constexpr size_t smem = collide_dyn_smem<D, R>(B::bx * B::by * B::bz);
     constexpr auto k = collide_stream_kernel<D, P, S, R, A>;
     configure<k>(smem);

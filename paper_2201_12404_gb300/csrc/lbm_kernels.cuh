@@ -122,6 +122,15 @@ moments_eos_kernel(DevDomain d) {
                                   B::bz);
 }
 
+// Pass 1 of a 3-D domain over consecutive nodes of a layer (FlatNode).
+template <int P, typename S, typename R, typename A>
+__global__ void __launch_bounds__(kFlatThreads, sizeof(R) == 8 ? 1 : (sizeof(S) == 2 ? LBM_K1_MINBLOCKS_F16 : LBM_K1_MINBLOCKS_F32))
+moments_eos_flat_kernel(DevDomain d) {
+  const FlatNode f(d);
+  if ((P == 1 || DevStorage<S>::value) && f.on_face) moments_eos_node<3, P, S, R, A, true>(d, f.x, f.y, f.z);
+  else moments_eos_node<3, P, S, R, A, false>(d, f.x, f.y, f.z);
+}
+
 }  // namespace lbm
 
 #include "lbm_collide.cuh"
