@@ -186,12 +186,12 @@ inline void fill_geometry(DevDomain& d, const lbm_params& p, int D, size_t pop_b
 
 // Which tile pass 1b takes.  2-D and float64: the small one where the large ones would
 // not fill the SMs once (128x128 2-D float32, passes 1 + 1b: 11.4 us small, 13.5 large;
-// the 800x10 column in float64 14.5 and 27 us).  3-D float32: the small one, 25 KB of
-// shared memory a block against 34, up to 160 large tiles per SM (19 million nodes).
-// Alone the large one gains there too (512x512x256: 2.10 ms against 2.14; 203x187x149:
-// 220 us against 221; 67x67x67: 32.0 against 30.3), but six large blocks take nearly all of
-// an SM's shared memory, and beside the other kernels of domains on other streams the SM
-// divides its memory anew for them: four cubes of 64 to 128 took 460 us a step against 380.
+// the 800x10 column in float64 14.5 and 27 us).  3-D float32: the small one, 23 KB of
+// shared memory a block against 34, up to 160 large tiles per SM (19 million nodes).  It
+// is the faster there (203x187x149: 188 us against 190) and loses above (512x512x256: 1.85 ms
+// against 1.82).  Six large blocks also take nearly all of an SM's shared memory, and
+// beside the kernels of domains on other streams the SM divides its memory anew for
+// them: four cubes of 64 to 128 took 460 us a step against 380 with tiles of 25 KB.
 template <typename T>
 inline long long tiles_of(const DevDomain& d) {
   return (long long)((d.nx + T::EX - 1) / T::EX) * ((d.ny + T::EY - 1) / T::EY) * ((d.nz + T::EZ - 1) / T::EZ);
