@@ -46,9 +46,8 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int* er
   return ok_s != 0;
 }
 
-// Minimum resident blocks per SM for the float32/float16 batch kernel.  Five
-// (51 registers, a few spilled) beat four (64, none) on the 16-job coexistence
-// batch: 17.7 against 16.7 GLUPS.
+// Minimum resident blocks per SM for the float32/float16 batch kernel: five (48 registers)
+// on the 16-job coexistence batch 89 us a step, four 92, six 96.
 #ifndef LBM_BATCH_MINBLOCKS_F32
 #define LBM_BATCH_MINBLOCKS_F32 5
 #endif

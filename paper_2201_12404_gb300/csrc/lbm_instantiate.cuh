@@ -41,7 +41,7 @@ struct Launch {
   // 203x187x149, 11%: 239.8, 239.5 and in float16 deviations 233, 255).  Pass 1 gains
   // up to 2.5 us of 26 and never lost more than 1%.
   static bool flat(const DevDomain& d) {
-    if (D == 2 || (long long)d.nx * d.ny >= 1 << 30 || d.nz > 65535) return false;
+    if (D == 2 || (long long)d.nx * d.ny >= 1 << 30 || (d.ny + B::by - 1) / B::by > 65535 || d.nz > 65535) return false;
     const long long lanes = (long long)((d.nx + B::bx - 1) / B::bx * B::bx) * ((d.ny + B::by - 1) / B::by * B::by);
     return 100 * lanes > 108 * ((long long)d.nx * d.ny);
   }

@@ -104,9 +104,8 @@ __global__ void __launch_bounds__(256) aux_density_kernel(DevDomain d, const dou
 }
 
 // Resident 64-thread blocks per SM asked of the register allocator in 3-D float32
-// arithmetic: 20 (48 registers) for float32 storage, passes 1 + 1b on the 203x187x149 impact
-// 215 us against 223 at 16 and 227 at 12; 16 (64) for float16 deviations, on 256x256x128
-// 319 us against 323 at 20 and 337 at 12.
+// arithmetic: 20 (48 registers) for float32 storage, passes 1 + 1b on 512x512x256 1.82 ms,
+// 1.85 at 16; 16 (64) for float16 deviations, on 256x256x128 271 us against 285 at 14.
 #ifndef LBM_K1_MINBLOCKS_F32
 #define LBM_K1_MINBLOCKS_F32 20
 #endif
