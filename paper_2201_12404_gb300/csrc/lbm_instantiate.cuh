@@ -140,8 +140,12 @@ struct Launch {
     return t.blocks;
   }
   static long long speed_partial(const DevDomain& d, const TileMaps& maps, double* partial, cudaStream_t s) {
-    if (partial) qflux_launch<kQfluxSpeed>(d, maps, partial, nullptr, s);
-    return maps.qtile_small ? tiles_of<QT<true>>(d) : tiles_of<QT<false>>(d);
+    const long long n = maps.qtile_small ? tiles_of<QT<true>>(d) : tiles_of<QT<false>>(d);
+    if (partial) {  // the word after the maxima, where their maximum goes in the end, starts the blocks at 0
+      cudaMemsetAsync(partial + n, 0, sizeof(double), s);
+      qflux_launch<kQfluxSpeed>(d, maps, partial, partial + n, s);
+    }
+    return n;
   }
   static void drop_on_film(const DevDomain& d, const lbm_drop_on_film& g, double rho_l, double rho_v, double* rho,
                            double* u, cudaStream_t s) {
