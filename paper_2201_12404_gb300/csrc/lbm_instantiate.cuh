@@ -136,6 +136,7 @@ struct Launch {
   };
   static int diag_partial(const DevDomain& d, int parity, double* partial, cudaStream_t s) {
     const Tiles t(d);
+    cudaMemsetAsync(partial + 5 * t.blocks, 0, sizeof(double), s);
     diag_partial_kernel<D, S><<<t.blocks, dim3(32, 8), 0, s>>>(d, parity, t.x, t.y, t.n, partial);
     return t.blocks;
   }

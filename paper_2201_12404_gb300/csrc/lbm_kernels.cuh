@@ -399,9 +399,11 @@ __global__ void bare_velocity_kernel(DevDomain d, const double* rho_in, double* 
 // partial layout: [block][5] = mass, jx, jy, jz, max|u|.
 //
 // Bound by the float64 pipe.  The totals are linear in the populations, so a thread sums
-// each of its Q slots over all of its nodes (one addition per population) and forms the moments once at the end; max|u| needs the moments of every
-// node, which float32 storage forms in float32 first and in float64 only where the speed
-// is not clearly below the largest this thread has seen.
+// each of its Q slots over all of its nodes (one addition per population, 388 us of the pipe
+// on 256x256x128) and forms the moments once at the end; max|u| needs the moments of
+// every node, which float32 storage forms in float32 first and in float64 only where the
+// speed is not clearly below the largest that any block has met (lbm_read_diag there 572 us;
+// 695 with each warp's own largest).
 // ---------------------------------------------------------------------------
 
 // g = (double)f, exactly.  For float32 by moving the fields of the bits where all Q values
@@ -437,7 +439,9 @@ __global__ void __launch_bounds__(256, 2) diag_partial_kernel(DevDomain d, int p
   __shared__ double sh[5][8];
   const int tid = threadIdx.x + 32 * threadIdx.y;
   double acc[Q], u2max = 0;
-  float top = 0.0f;  // largest float32 speed squared this warp has met
+  float top = 0.0f;  // largest float32 speed squared that this warp knows of
+  // shared by the grid: the bits of the largest so far, after the partials
+  volatile unsigned* top_all = (unsigned*)(partial + 5 * (long long)gridDim.x);
 #pragma unroll
   for (int i = 0; i < Q; ++i) acc[i] = 0;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -446,6 +450,8 @@ __global__ void __launch_bounds__(256, 2) diag_partial_kernel(DevDomain d, int p
     L f[Q];
     double g[Q];
     float u2f = 0.0f;
+    unsigned known = 0;
+    if constexpr (sizeof(L) == 4) known = *top_all;
     if (in) {
       gather<D, S, L>(d, parity, x, y, z, f);
       if constexpr (sizeof(L) == 4) {
@@ -459,7 +465,9 @@ __global__ void __launch_bounds__(256, 2) diag_partial_kernel(DevDomain d, int p
     }
     if constexpr (sizeof(L) == 4) {
       // non-negative floats order as their bits; a NaN is above them all
-      top = fmaxf(top, __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(u2f))));
+      const float others = __uint_as_float(known);
+      top = fmaxf(fmaxf(top, others), __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(u2f))));
+      if (top > others && threadIdx.x == 0) atomicMax((unsigned*)top_all, __float_as_uint(top));
       in = in && !(u2f < 0.999f * top);
     }
     if (in) {
