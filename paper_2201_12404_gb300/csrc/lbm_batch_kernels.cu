@@ -65,11 +65,17 @@ __global__ void __launch_bounds__(BX * BY, sizeof(R) == 4 ? LBM_BATCH_MINBLOCKS_
   R* s_h = (R*)smem_dyn;
   const int tid = threadIdx.x + BX * threadIdx.y;
   const int lo = (int)((long long)a.ntiles * blockIdx.x / gridDim.x), hi = (int)((long long)a.ntiles * (blockIdx.x + 1) / gridDim.x);
+  int job0 = 0;  // the job of tile lo, by bisection
+  for (int n = a.njobs; n > 1;) {
+    const int half = n >> 1;
+    if (a.tiles[job0 + half].first <= lo) { job0 += half; n -= half; }
+    else n = half;
+  }
   int job = -1, first = 0, end = 0, ntx = 1, parity = 0;  // of the job in d
   // The job of tile t into d (a block barrier when it changes); every thread calls it.
   auto select = [&](int t) {
     if (job >= 0 && t >= first && t < end) return;
-    if (job < 0 || t < first) job = 0;
+    if (job < 0 || t < first) job = job0;
     while (t >= a.tiles[job + 1].first) ++job;
     first = a.tiles[job].first;
     end = a.tiles[job + 1].first;
