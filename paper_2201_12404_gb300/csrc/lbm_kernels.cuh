@@ -402,9 +402,20 @@ __global__ void bare_velocity_kernel(DevDomain d, const double* rho_in, double* 
 // each of its Q slots over all of its nodes (one addition per population, 388 us of the pipe
 // on 256x256x128) and forms the moments once at the end; max|u| needs the moments of
 // every node, which float32 storage forms in float32 first and in float64 only where the
-// speed is not clearly below the largest that any block has met (lbm_read_diag there 572 us;
-// 695 with each warp's own largest).
+// node may be the fastest: slower_than_top is right whatever the order in which the blocks
+// meet their nodes (lbm_read_diag there 576 us; 695 with each warp's own largest).
 // ---------------------------------------------------------------------------
+
+// Whether a node is slower than one met before, from float32 speeds squared: u2f of this
+// node, top the largest so far.  Both nodes have populations >= 0, so a momentum of five
+// additions deep is within 5 2^-24 rho of the exact one (the vector within 5.2e-7 rho) and
+// rho within 6 2^-24 of itself; with the roundings of the quotient a float32 speed is within
+// 6e-7 + 1e-6 |u| of the exact one.  A relative margin alone, as wide as 0.999 of the
+// square, would pass over the fastest node below speeds of 1e-3.
+__device__ __forceinline__ bool slower_than_top(float u2f, float top) {
+  const float least = fmaf(sqrtf(top), 0.9999f, -2e-6f);
+  return least > 0.0f && u2f < least * least;
+}
 
 // g = (double)f, exactly.  For float32 by moving the fields of the bits where all Q values
 // are normal numbers: the float64 pipe, which also runs the conversion instruction, sets
@@ -450,6 +461,7 @@ __global__ void __launch_bounds__(256, 2) diag_partial_kernel(DevDomain d, int p
     L f[Q];
     double g[Q];
     float u2f = 0.0f;
+    bool known_speed = false;  // u2f holds to within the bound of slower_than_top
     unsigned known = 0;
     if constexpr (sizeof(L) == 4) known = *top_all;
     if (in) {
@@ -457,18 +469,22 @@ __global__ void __launch_bounds__(256, 2) diag_partial_kernel(DevDomain d, int p
       if constexpr (sizeof(L) == 4) {
         NodeMoments<float> m;
         row_moments<D, float>(f, m);
-        u2f = (m.jx * m.jx + m.jy * m.jy + m.jz * m.jz) / (m.rho * m.rho);
+        unsigned signs = 0;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) signs |= __float_as_uint(f[i]);
+        known_speed = (int)signs >= 0 && m.rho > 1e-15f && m.rho < 1e15f;  // (a NaN is not)
+        if (known_speed) u2f = (m.jx * m.jx + m.jy * m.jy + m.jz * m.jz) / (m.rho * m.rho);
       }
       widen<Q>(f, g);
 #pragma unroll
       for (int i = 0; i < Q; ++i) acc[i] += g[i];
     }
     if constexpr (sizeof(L) == 4) {
-      // non-negative floats order as their bits; a NaN is above them all
+      // non-negative floats order as their bits
       const float others = __uint_as_float(known);
       top = fmaxf(fmaxf(top, others), __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(u2f))));
       if (top > others && threadIdx.x == 0) atomicMax((unsigned*)top_all, __float_as_uint(top));
-      in = in && !(u2f < 0.999f * top);
+      in = in && !(known_speed && slower_than_top(u2f, top));
     }
     if (in) {
       NodeMoments<double> m;
