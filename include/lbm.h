@@ -102,8 +102,7 @@ typedef struct {
   int32_t gamma_mode;   /* lbm_gamma_mode */
   double gamma_value;   /* used when gamma_mode == LBM_GAMMA_FIXED */
   /* FP32 path only: 0 = Peng-Robinson pressure in float32 everywhere,
-   * 1 = beyond float32 (pairs of float32, or float64), rounded once, where rho lies
-   *     inside the interface band (default),
+   * 1 = in float64 where rho lies inside the interface band (default),
    * 2 = float64 everywhere. */
   int32_t eos_fp64;
   void* stream;         /* cudaStream_t to run on; NULL = a stream the library creates */
