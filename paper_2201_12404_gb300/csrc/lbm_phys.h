@@ -108,11 +108,10 @@ inline void fill_phys(DevDomain& d, const lbm_params& p, int D) {
   // and M = 3 (1 - t)(1 + 2t - t^2).
   const double num[4] = {3 * e.RT - 1, (6 * e.RT - 1) * e.b - 3 * e.aalpha, ((3 - 3 * e.RT) * e.b + 3 * e.aalpha) * e.b,
                          -e.b * e.b * e.b};
-  const double den[4] = {3, 3 * e.b, -9 * e.b * e.b, 3 * e.b * e.b * e.b};
-  for (int k = 0; k < 4; ++k) {
-    d.eos_num[k].x = (float)num[k]; d.eos_num[k].y = (float)(num[k] - d.eos_num[k].x);
-    d.eos_den[k].x = (float)den[k]; d.eos_den[k].y = (float)(den[k] - d.eos_den[k].x);
-  }
+  const double den[3] = {3 * e.b, -9 * e.b * e.b, 3 * e.b * e.b * e.b};  // after the constant 3
+  auto split = [](double c) { return float2{(float)c, (float)(c - (float)c)}; };
+  for (int k = 0; k < 4; ++k) d.eos_num[k] = split(num[k]);
+  for (int k = 0; k < 3; ++k) d.eos_den[k] = split(den[k]);
   // Error of psi_banded, u = 2^-24.  A cubic by three pair steps: each rounds three tails of at
   // most 7u of the sum S of the term magnitudes so far, 18 u^2 S, so 2^-42 S in all.  The
   // quotient's and the product's second terms 38 u^2 v, v = |P - P0| = psi^2; the root's, from an
