@@ -217,7 +217,8 @@ lbm_status lbm_init_drop_on_film(lbm_handle h, const lbm_drop_on_film* g);
  * (the exact-difference-method velocity that lbm_read_macroscopic returns,
  * the velocity whose maximum the paper reports as the spurious current,
  * Sec. 3.1.2), reduced on the GPU: one pass-1 launch for the current state,
- * one reduction.  A state with a non-finite speed gives +inf.  Synchronising. */
+ * one reduction.  A state with a non-finite speed gives +inf.  LBM_ERR_TIMEOUT when a
+ * bounded device-side wait has given up.  Synchronising. */
 lbm_status lbm_max_speed(lbm_handle h, double* max_u);
 
 /* Interface thickness W = (rho_liquid - rho_vapour) / max |grad rho| of the

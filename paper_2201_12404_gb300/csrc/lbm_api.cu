@@ -327,21 +327,26 @@ double bisect_p(const EosCoeffs& e, double target, double lo, double hi) {
 }
 
 // Pass 1 for the current state, then block maxima (partial(buf, stream), which returns
-// their number and launches nothing for a null buffer) and their maximum in *out.
+// their number and launches nothing for a null buffer) and their maximum in *out.  A block
+// whose TMA tile did not arrive stores no maximum: the error word is read with the result.
+// (Instability is left to the calls that report it: the readings serve to look at such states.)
 template <typename Partial>
 lbm_status reduce_max(lbm_handle h, Partial partial, double* out) {
   lbm_status st = refresh_aux(h);
   if (st != LBM_OK) return st;
   const long long nb = partial(nullptr);
   double* buf = nullptr;
-  LBM_CUDA(h, scratch_alloc(h, &buf, (size_t)(nb + 1) * sizeof(double)));
+  LBM_CUDA(h, scratch_alloc(h, &buf, (size_t)(nb + 2) * sizeof(double)));
   partial(buf);
-  lbm::launch_max_final(buf, nb, buf + nb, h->stream);
+  lbm::launch_max_final(buf, nb, h->dev.flags, buf + nb, h->stream);
   h->launches += 2;
   LBM_CUDA(h, cudaGetLastError());
-  LBM_CUDA(h, cudaMemcpyAsync(out, buf + nb, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  double res[2];
+  LBM_CUDA(h, cudaMemcpyAsync(res, buf + nb, sizeof(res), cudaMemcpyDeviceToHost, h->stream));
   LBM_CUDA(h, cudaFreeAsync(buf, h->stream));
   LBM_CUDA(h, cudaStreamSynchronize(h->stream));
+  if ((st = flags_status(h, (unsigned)res[1] & ~1u)) != LBM_OK) return st;
+  *out = res[0];
   return LBM_OK;
 }
 

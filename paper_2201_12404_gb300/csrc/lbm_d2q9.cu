@@ -9,8 +9,8 @@ const Ops ops_d2q9_fp16dev = Launch<2, __half, float, float>::table();
 void launch_diag_final(const double* partial, int nblocks, double* out, cudaStream_t s) {
   diag_final_kernel<<<1, dim3(32, 5), 0, s>>>(partial, nblocks, out);
 }
-void launch_max_final(const double* partial, long long n, double* out, cudaStream_t s) {
-  max_final_kernel<<<1, 1024, 0, s>>>(partial, n, out);
+void launch_max_final(const double* partial, long long n, const unsigned* flags, double* out, cudaStream_t s) {
+  max_final_kernel<<<1, 1024, 0, s>>>(partial, n, flags, out);
 }
 int diag_blocks() { return kDiagBlocks; }
 }  // namespace lbm

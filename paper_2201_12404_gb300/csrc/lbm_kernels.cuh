@@ -528,11 +528,14 @@ static __global__ void diag_final_kernel(const double* partial, int nblocks, dou
   if (threadIdx.x == 0) out[k] = v;
 }
 
-// Largest of n partial maxima, by one block of 1024 threads.
-static __global__ void __launch_bounds__(1024) max_final_kernel(const double* partial, long long n, double* out) {
+// Largest of n partial maxima, by one block of 1024 threads, to out[0]; the domain's error word
+// to out[1], so that one copy tells the host whether a block gave up its wait.
+static __global__ void __launch_bounds__(1024) max_final_kernel(const double* partial, long long n, const unsigned* flags,
+                                                                double* out) {
   double v = 0;
   for (long long b = threadIdx.x; b < n; b += 1024) v = fmax(v, partial[b]);
   block_max_store<1024>(threadIdx.x, v, out, 0);
+  if (threadIdx.x == 0) out[1] = (double)*flags;
 }
 
 }  // namespace lbm

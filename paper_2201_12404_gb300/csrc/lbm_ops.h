@@ -249,8 +249,8 @@ inline bool make_tile_maps(TileMaps* m, const DevDomain& d, int D, size_t elem_b
 // Blocks of diag_partial.
 int diag_blocks();
 // Final fixed-order reductions (lbm_d2q9.cu): out[5] of the totals' partials, out[0] the
-// largest of n block maxima.
+// largest of n block maxima and out[1] the error word.
 void launch_diag_final(const double* partial, int nblocks, double* out, cudaStream_t s);
-void launch_max_final(const double* partial, long long n, double* out, cudaStream_t s);
+void launch_max_final(const double* partial, long long n, const unsigned* flags, double* out, cudaStream_t s);
 
 }  // namespace lbm
