@@ -314,7 +314,8 @@ __global__ void drop_on_film_kernel(DevDomain d, double R, double film, double g
 // the ghost layer supplies the wrapped or mirrored neighbours): kDiagBlocks blocks at
 // most, each over every gridDim-th tile of 32 x 8 nodes, one partial maximum per block.
 // Float64 is 58 times slower than float32, so a warp differences in float64 only the
-// nodes whose float32 gradient is not clearly below the largest it has met.
+// nodes whose float32 gradient is not clearly below the largest it has met (1e-35 off the
+// bound on its square: squares below the normal numbers have lost their relative precision).
 // ---------------------------------------------------------------------------
 constexpr int kDiagBlocks = 152 * 6;
 
@@ -341,7 +342,7 @@ __global__ void __launch_bounds__(256) grad_partial_kernel(DevDomain d, int ntx,
     }
     // non-negative floats order as their bits; a NaN is above them all
     top = fmaxf(top, __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(g2f))));
-    if (in && !(g2f < 0.99f * top)) {
+    if (in && !(g2f < fmaf(0.99f, top, -1e-35f))) {
       double g2 = 0;
 #pragma unroll
       for (int a = 0; a < D; ++a) {
