@@ -112,18 +112,19 @@ inline void fill_phys(DevDomain& d, const lbm_params& p, int D) {
   auto split = [](double c) { return float2{(float)c, (float)(c - (float)c)}; };
   for (int k = 0; k < 4; ++k) d.eos_num[k] = split(num[k]);
   for (int k = 0; k < 3; ++k) d.eos_den[k] = split(den[k]);
-  // Error of psi_banded, u = 2^-24.  A cubic by three pair steps: each rounds three tails of at
-  // most 7u of the sum S of the term magnitudes so far, 18 u^2 S, so 2^-42 S in all.  The
-  // quotient's and the product's second terms 38 u^2 v, v = |P - P0| = psi^2; the root's, from an
-  // approximation within 2^-22.9 and one step of the residual, 95 u^2 psi.  With half the
-  // relative errors of v for psi that is psi (2^-41 + 2^-43 S_M/M) + 2^-43 rho (S_N/M) / psi, over
-  // which the bound holds a factor of two.  S at the upper end of the band, M (rising, then
-  // falling in t) at one end; S_N also covers the terms of the float64 pressure.
+  // Error of psi_banded, u = 2^-24.  A cubic's three pair steps round three tails each, of at most
+  // 3u, 5u and 7u of the sum S of the term magnitudes: 40 u^2 S with the coefficients' own.  The
+  // quotient's and the product's second terms, from a reciprocal within 2u: 38 u^2 v, v = |P - P0| =
+  // psi^2.  The root, from an approximation within 2^-22.9 and one residual step: 68 u^2 psi; the
+  // ends of the interval 6 u^2 psi.  With half the relative errors of v for psi that is
+  // psi u^2 (93 + 20 S_M/M) + u^2 20 rho (S_N/M) / psi, rounded up.  S at the upper end of the
+  // band, M (rising, then falling in t) at one end; S_N also covers the terms of the float64
+  // pressure, whose own error is a thousandth of this.
   const double t = e.b * pd.band_hi, t2 = (1 + t) * (1 + t);
   const double S_M = 3 + 3 * t + 9 * t * t + 3 * t * t * t, M = std::fmin(3.0, 3 * (1 - t) * (1 + 2 * t - t * t));
   const double S_N = 3 * e.RT * t2 + 3 * e.aalpha * pd.band_hi * (1 + t) + (1 + t) * t2;
-  d.eos_err.x = (float)(std::ldexp(1.0, -40) * (1 + S_M / M / 4));
-  d.eos_err.y = (float)(std::ldexp(1.0, -42) * pd.band_hi * S_N / M);
+  d.eos_err.x = (float)(std::ldexp(1.0, -48) * (100 + 21 * S_M / M));
+  d.eos_err.y = (float)(std::ldexp(1.0, -48) * 21 * S_N / M);
   // The pairs need the poles outside the band and products well inside float32's range;
   // every calibrated parameter set of the equation is (b rho < 1, the rest of order one).
   auto moderate = [](double x) { return std::fabs(x) > 1e-6 && std::fabs(x) < 1e6; };
