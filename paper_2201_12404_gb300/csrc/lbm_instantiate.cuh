@@ -33,11 +33,11 @@ struct Launch {
     }
     return dim3(gx, ty, (d.nz + B::bz - 1) / B::bz);
   }
-  // Whether passes 1 and 2 take consecutive nodes of a layer instead of tiles: where tiles
-  // would idle more than 8% of their lanes.  Without tiles pass 2 reads q from global
+  // Whether passes 1 and 2 take consecutive nodes of a layer instead of tiles: where the tiles
+  // have over 8% more lanes than the layer has nodes.  Without tiles pass 2 reads q from global
   // memory, which costs more than it gives where few lanes idle (pass 2 of 512x512x256
   // in float32: 2.69 ms against 2.58, of 128^3 90.0 us against 87.6) and less elsewhere
-  // (67^3, 46% idle: 16.4 us against 19.4; 107^3, 21%: 54.5, 57.5; 85^3, 14%: 26.6, 28.5;
+  // (67^3, 45% more: 16.4 us against 19.4; 107^3, 21%: 54.5, 57.5; 85^3, 14%: 26.6, 28.5;
   // 203x187x149, 11%: 239.8, 239.5 and in float16 deviations 233, 255).  Pass 1 gains
   // up to 2.5 us of 26 and never lost more than 1%.
   static bool flat(const DevDomain& d) {
