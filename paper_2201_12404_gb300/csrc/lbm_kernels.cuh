@@ -105,16 +105,23 @@ __global__ void __launch_bounds__(256) aux_density_kernel(DevDomain d, const dou
 
 // Resident 64-thread blocks per SM asked of the register allocator in 3-D float32
 // arithmetic: 20 (48 registers) for float32 storage, passes 1 + 1b on 512x512x256 1.82 ms,
-// 1.85 at 16; 16 (64) for float16 deviations, on 256x256x128 271 us against 285 at 14.
+// 1.85 at 16; 16 (64) for float16 deviations, on 256x256x128 271 us against 285 at 14.  2-D:
+// 16 128-thread blocks (32 registers) for float32 storage, 2048x1024 40.5 us, 40.8 with 37.
 #ifndef LBM_K1_MINBLOCKS_F32
 #define LBM_K1_MINBLOCKS_F32 20
 #endif
 #ifndef LBM_K1_MINBLOCKS_F16
 #define LBM_K1_MINBLOCKS_F16 16
 #endif
+#ifndef LBM_K1_MINBLOCKS_F32_2D
+#define LBM_K1_MINBLOCKS_F32_2D 16
+#endif
 template <int D, int P, typename S, typename R, typename A>
 __global__ void __launch_bounds__(Blocks<D, R>::bx * Blocks<D, R>::by * Blocks<D, R>::bz,
-                                  D == 3 && sizeof(R) == 4 ? (sizeof(S) == 2 ? LBM_K1_MINBLOCKS_F16 : LBM_K1_MINBLOCKS_F32) : 1)
+                                  sizeof(R) == 8   ? 1
+                                  : D == 2         ? (sizeof(S) == 2 ? 1 : LBM_K1_MINBLOCKS_F32_2D)
+                                  : sizeof(S) == 2 ? LBM_K1_MINBLOCKS_F16
+                                                   : LBM_K1_MINBLOCKS_F32)
 moments_eos_kernel(DevDomain d) {
   using B = Blocks<D, R>;
   moments_eos_tile<D, P, S, R, A>(d, blockIdx.x * B::bx, tile_y<D>() * B::by, D == 3 ? blockIdx.z * B::bz : 0, B::bx, B::by,
