@@ -47,16 +47,17 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int* er
 }
 
 // Minimum resident blocks per SM for the float32/float16 batch kernel: five (48 registers)
-// on the 16-job coexistence batch 89 us a step, four 92, six 96.
+// on the 16-job coexistence batch 90 us a step, four 95, six 94.
 #ifndef LBM_BATCH_MINBLOCKS_F32
 #define LBM_BATCH_MINBLOCKS_F32 5
 #endif
 // Every block takes a consecutive share of the tiles: they are mostly of one job, whose
 // description the block keeps in shared memory through all passes and steps, and a tile's
-// neighbours are its own (16-job coexistence batch, float32: 88 us a step; 106 with the
-// tiles dealt out one by one and a list read per tile, 99 with shared descriptions alone,
-// 101 with tiles drawn from a counter).  Bound by latency: the passes take 20, 25 and 29 us
-// and the wait at each barrier 8 to 11, most of it for the blocks with one tile more.
+// neighbours are its own (16-job coexistence batch, float32: 88 us a step when written, 90 now;
+// 106 with the tiles dealt out one by one and a list read per tile, 99 with shared
+// descriptions alone, 101 with tiles drawn from a counter).  Bound by latency: the passes took
+// 20, 25 and 29 of the 88 us and the wait at each barrier 8 to 11, most of it for the blocks
+// with one tile more.
 template <int BX, int BY, typename S, typename R, typename A>
 __global__ void __launch_bounds__(BX * BY, sizeof(R) == 4 ? LBM_BATCH_MINBLOCKS_F32 : 1) batch_persistent_kernel(BatchArgs a) {
   __shared__ __align__(128) Two<A> s_aux[QTileShape<2, BX, BY, 1>::HX * QTileShape<2, BX, BY, 1>::HY];
