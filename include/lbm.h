@@ -66,7 +66,7 @@ typedef enum { LBM_D2Q9 = 0, LBM_D3Q27 = 1 } lbm_lattice;
 /* Storage and arithmetic of the populations.
  * LBM_FP64: stored and computed in float64 (the GPU reference path).
  * LBM_FP32: stored and computed in float32; float64 only in the Peng-Robinson
- *           pressure inside the interface band and in the gamma ratio.
+ *           pressure inside the interface band (eos_fp64).
  * LBM_FP16DEV: stored as float16 deviations f_i/(w_i rho_w) - 1, rho_w the
  *           density of the node that wrote the slot (kept per node, one float32
  *           per node and parity); computed in float32 like LBM_FP32. */
